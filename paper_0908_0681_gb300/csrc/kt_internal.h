@@ -5,6 +5,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <vector_types.h>
+
 #include "../../include/kt.h"
 
 namespace kt {
@@ -53,6 +55,21 @@ struct DevModel {
   const int32_t *blk_evoff;
   const float *blk_evec32;
   const float *blk_evec32lo;
+
+  // traces in the block eigenbasis (kt_eig.cuh)
+  int eig;                    // how vectors are held (EIG_PAIR, EIG_F64), -1: Krylov propagation only
+  int key_mask;               // bits of the singly-occupied mask that the block keys use (0: sector blocks)
+  const int16_t *key_lut;     // [(n_orb + 1)^2 << n_orb] block of (n_up, n_dn, mask), -1 if none
+  const int32_t *blk_key;     // [n_blocks] n_up + 1024 n_dn + (mask << 20)
+  const int32_t *kept_key;    // [n_kept] the key of the kept state's block
+  const int32_t *kept_row;    // [n_kept] its eigenvalue index inside the block
+  const int4 *eig_op;         // [n_blocks * nf * 2] {first 16-byte vector of the matrix, blk_off of the target |
+                              //   rows of the source << 16 | rows of the target << 22, target, 0}
+  const double *eig_base;     // [n_blocks] s_b - E0
+  const void *eig_lam;        // [n_states] (lambda_k - lambda_0) log2 e per global row: float pairs, or FP64
+  const void *eig_tab;        // 2^(j/32) as 32 float pairs, or 2^(j/128) as 128 FP64
+  const void *eig_mat;        // operator matrices between block eigenbases, rows padded to 16 bytes
+  const double *blk_evec64;   // eigenvectors in FP64, laid out as blk_evec32
 
   const int32_t *kept_blk;    // [n_kept]
   const double *kept_e;       // [n_kept] E - E0
@@ -105,8 +122,9 @@ struct Workspace {
 // state right after operator i-1, at its time; position 0 is the kept state at
 // tau = 0 and is not stored) and backward states at reverse slot K - e (the bra
 // including operators e .. K-1, at the time of operator e; reverse slot 0 is the kept
-// state at beta). Entries are normalised vectors with a log-weight and their block
-// (-1: the state is zero). f[item] and gr[item] bound the valid forward slots
+// state at beta). Entries are vectors with a log-weight and their block (-1: the state is
+// zero): components on the block's eigenvectors for models with traces in the block
+// eigenbasis (DevModel.eig >= 0), normalised vectors in the occupation basis otherwise. f[item] and gr[item] bound the valid forward slots
 // [0, f] and reverse slots [0, gr]. The scratch arrays hold one step's tentative
 // states (inside the edited window) until the accept decision.
 struct CacheView {
@@ -146,6 +164,7 @@ int kernel_dmax_for(int d_max);    // 0 if no variant fits
 int kernel_pmax_for(int kernel_dmax);
 int kernel_groups_for(int kernel_dmax, int *out, int cap);  // lane-group sizes compiled for this row capacity
 int default_group_for(int kernel_dmax, int precision);
+int default_eig_group_for(int kernel_dmax);  // the same for traces in the block eigenbasis
 
 // Optional CUDA events recorded at the 5 stage boundaries of one pipeline call.
 struct StageEvents {
@@ -161,6 +180,24 @@ int launch_pipeline(const DevModel &m, int precision, int kernel_dmax, int group
                     const int8_t *cur_sign, const double *cur_logabs, int8_t *sign, double *logv, int32_t *status,
                     kt_stats *stats, const Workspace &ws, void *stream, const StageEvents *timing,
                     double *obs = nullptr);
+
+// Operator matrices between the block eigenbases (eig_op, eig_mat) from the eigenvectors,
+// on the default stream. Returns a CUDA error code.
+int build_eig_matrices(const DevModel &m);
+// The whole call in the block eigenbasis (m.eig >= 0), one kernel: arguments as launch_pipeline.
+int launch_eig_pipeline(const DevModel &m, int kernel_dmax, int group_lanes, const SeqView &seq, const MoveView *moves,
+                        const int8_t *cur_sign, const double *cur_logabs, int8_t *sign, double *logv, int32_t *status,
+                        const Workspace &ws, void *stream, double *obs);
+
+// The cached calls in the block eigenbasis, one kernel each: arguments as launch_cached_pipeline,
+// launch_cache_build and launch_cached_measure.
+int launch_eig_cached(const DevModel &m, int kernel_dmax, const SeqView &seq, const MoveView &moves,
+                      const int8_t *cur_sign, const double *cur_logabs, int8_t *sign, double *logv, int32_t *status,
+                      const Workspace &ws, const CacheView &cache, bool write, void *stream);
+int launch_eig_build(const DevModel &m, int kernel_dmax, const SeqView &seq, const Workspace &ws,
+                     const CacheView &cache, void *stream);
+int launch_eig_measure(const DevModel &m, int kernel_dmax, const SeqView &seq, int8_t *sign, double *logv,
+                       int32_t *status, double *obs, const Workspace &ws, const CacheView &cache, void *stream);
 
 // The trace-ratio pipeline of the sweep's cached mode: validation and edit, the
 // per-item plan (pruning, the stretch between valid cached states), the cached

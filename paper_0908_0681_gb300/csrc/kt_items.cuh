@@ -1412,15 +1412,27 @@ __global__ void __launch_bounds__(256, KT_MIN_CTAS(VT)) items_kernel(DevModel M,
 // One cache entry: the unit's normalised vector, its log-weight as (additive part
 // less the binary exponent of the normalisation product, mantissa of that product)
 // so that no logarithm is taken per operator, and its block (-1: the state is zero).
-template <typename VT, int G, int DMAX, int PMAX>
-__device__ __forceinline__ void store_entry(VT *vec, double2 *lg, int32_t *bk, size_t e, int dv,
+// For models with traces in the block eigenbasis (M.eig >= 0) the other kernels keep the
+// components on the block's eigenvectors: the instances that count work, the only ones that
+// such a model runs on its cache, change the basis at each entry.
+template <int OPT, typename VT, int G, int DMAX, int PMAX>
+__device__ __forceinline__ void store_entry(const DevModel &M, VT *vec, double2 *lg, int32_t *bk, size_t e, int dv,
                                             Unit<VT, G, DMAX, PMAX> &u, bool zero) {
   constexpr int R = Unit<VT, G, DMAX, PMAX>::R;
   if (!zero) {
 #pragma unroll
     for (int j = 0; j < R; ++j) {
       const int r = u.gl + G * j;
-      if (r < u.dim) vec[e * dv + r] = u.Q(0, r);
+      if (r < u.dim) {
+        VT x = u.Q(0, r);
+        if ((OPT & KT_OPT_STATS) && M.eig >= 0) {
+          const double *V = M.blk_evec64 + __ldg(M.blk_evoff + u.b) + (size_t)r * u.dim;
+          double a = 0.0;
+          for (int i = 0; i < u.dim; ++i) a = fma(__ldg(V + i), (double)u.Q(0, i), a);
+          x = (VT)a;
+        }
+        vec[e * dv + r] = x;
+      }
     }
   }
   if (u.gl == 0) {
@@ -1429,7 +1441,7 @@ __device__ __forceinline__ void store_entry(VT *vec, double2 *lg, int32_t *bk, s
   }
 }
 
-template <typename VT, int G, int DMAX, int PMAX>
+template <int OPT, typename VT, int G, int DMAX, int PMAX>
 __device__ __forceinline__ bool load_entry(const DevModel &M, const VT *vec, const double2 *lg, const int32_t *bk,
                                            size_t e, int dv, Unit<VT, G, DMAX, PMAX> &u) {
   constexpr int R = Unit<VT, G, DMAX, PMAX>::R;
@@ -1437,15 +1449,40 @@ __device__ __forceinline__ bool load_entry(const DevModel &M, const VT *vec, con
   if (b < 0) return false;
   u.b = b;
   u.dim = __ldg(M.blk_dim + b);
-#pragma unroll
-  for (int j = 0; j < R; ++j) {
-    const int r = u.gl + G * j;
-    if (r < u.dim) u.Q(0, r) = __ldcg(vec + e * dv + r);
-  }
   const double2 l = __ldcg(lg + e);
   u.Ladd = l.x;
   u.Linv.m = l.y;
   u.Linv.e = 0;
+  VT v[R];
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const int r = u.gl + G * j;
+    v[j] = r < u.dim ? __ldcg(vec + e * dv + r) : VT(0);
+  }
+  if ((OPT & KT_OPT_STATS) && M.eig >= 0) {
+    const double *V = M.blk_evec64 + __ldg(M.blk_evoff + b);
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const int r = u.gl + G * j;
+      if (r < u.dim) u.Q(0, r) = v[j];
+    }
+    __syncwarp(u.gm);
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const int r = u.gl + G * j;
+      double a = 0.0;
+      if (r < u.dim)
+        for (int k = 0; k < u.dim; ++k) a = fma(__ldg(V + (size_t)k * u.dim + r), (double)u.Q(0, k), a);
+      v[j] = (VT)a;
+    }
+    __syncwarp(u.gm);
+    if (!normalize_rows<VT, G, R>(v, u.gl, u.dim, u.gm, u.Linv)) return false;
+  }
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const int r = u.gl + G * j;
+    if (r < u.dim) u.Q(0, r) = v[j];
+  }
   __syncwarp(u.gm);
   return true;
 }
@@ -1524,7 +1561,7 @@ __global__ void __launch_bounds__(256, KT_MIN_CTAS(VT)) items_cached_kernel(DevM
       }
       __syncwarp(gm);
     } else {
-      vanished = !load_entry(M, (const VT *)(fwd ? C.fvec : C.bvec), fwd ? C.flog : C.blog, fwd ? C.fblk : C.bblk,
+      vanished = !load_entry<OPT>(M, (const VT *)(fwd ? C.fvec : C.bvec), fwd ? C.flog : C.blog, fwd ? C.fblk : C.bblk,
                              eb + (fwd ? start : Kn - start), dv, u);
     }
     const int n_ops = build ? Kn : (fwd ? m - y : x - m);
@@ -1554,7 +1591,7 @@ __global__ void __launch_bounds__(256, KT_MIN_CTAS(VT)) items_cached_kernel(DevM
         VT *vec = (VT *)(fwd ? (out ? C.fvec : C.sfvec) : (out ? C.bvec : C.sbvec));
         double2 *lg = fwd ? (out ? C.flog : C.sflog) : (out ? C.blog : C.sblog);
         int32_t *bk = fwd ? (out ? C.fblk : C.sfblk) : (out ? C.bblk : C.sbblk);
-        store_entry(vec, lg, bk, e, dv, u, vanished);
+        store_entry<OPT>(M, vec, lg, bk, e, dv, u, vanished);
       }
     }
     // a measurement stores states of the current configuration: the valid range grows

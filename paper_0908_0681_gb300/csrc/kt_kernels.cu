@@ -54,7 +54,6 @@ using namespace dev;
 // ---------------------------------------------------------------------------
 __global__ void prep_kernel(DevModel M, SeqView S, MoveView mv, int has_moves, const int8_t *cur_sign, Workspace ws,
                             kt_stats *stats) {
-  // one warp per walker: the lanes read consecutive operators (coalesced) and decide by ballot
   const int lane = threadIdx.x & 31;
   const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -64,82 +63,8 @@ __global__ void prep_kernel(DevModel M, SeqView S, MoveView mv, int has_moves, c
     ws.counters[3] = 0;
   }
   if (w >= S.n) return;
-  const int o = S.offsets[w], K = S.lens ? S.lens[w] : S.offsets[w + 1] - o;
-  int st = KT_OK;
-  int4 d = make_int4(-1, 0, 0, K);
-  if (K < 0) {
-    st = KT_EINVAL;
-  } else if (!S.trusted) {
-    // times non-decreasing from 0 and below beta, flavors and daggers in range
-    double carry = 0.0;
-    for (int base = 0; base < K; base += 32) {
-      const int i = base + lane;
-      double t = 0.0;
-      int f = 0, g = 0;
-      if (i < K) {
-        t = __ldg(S.tau + o + i);
-        f = __ldg(S.flavor + o + i);
-        g = __ldg(S.dagger + o + i);
-      }
-      double prev = __shfl_up_sync(FULL, t, 1);
-      if (lane == 0) prev = carry;
-      const bool bad = i < K && (!(t >= prev) || !(t < M.beta) || f >= M.nf || g > 1);
-      if (__any_sync(FULL, bad)) {
-        st = KT_EINVAL;
-        break;
-      }
-      carry = __shfl_sync(FULL, t, 31);
-    }
-  }
-  if (has_moves && st == KT_OK) {
-    const int kind = mv.kind[w], f = mv.flavor[w];
-    if (f >= M.nf) {
-      st = KT_EINVAL;
-    } else if (kind == 0) {
-      const double td = mv.t_dag[w], ta = mv.t_ann[w];
-      if (!(td >= 0.0 && td < M.beta && ta >= 0.0 && ta < M.beta)) {
-        st = KT_EINVAL;
-      } else {
-        // insertion points: the number of operators at or before each new time (the sorted
-        // sequence's upper bound)
-        const double tA = td < ta ? td : ta, tB = td < ta ? ta : td;
-        int pa = 0, pb = 0;
-        for (int base = 0; base < K; base += 32) {
-          const int i = base + lane;
-          const double t = i < K ? __ldg(S.tau + o + i) : 0.0;
-          pa += __popc(__ballot_sync(FULL, i < K && t <= tA));
-          pb += __popc(__ballot_sync(FULL, i < K && t <= tB));
-        }
-        d = make_int4(0, pa, pb, K + 2);
-      }
-    } else if (kind == 1) {
-      const int r = mv.rem_idx[w];
-      if (r < 0 || r >= K || S.flavor[o + r] != f) {
-        st = KT_EINVAL;
-      } else {
-        // its partner: the next operator of the flavor after r, cyclically
-        int j = -1;
-        for (int base = r + 1; base < K && j < 0; base += 32) {
-          const int i = base + lane;
-          const unsigned m = __ballot_sync(FULL, i < K && __ldg(S.flavor + o + i) == f);
-          if (m) j = base + __ffs(m) - 1;
-        }
-        for (int base = 0; base < r && j < 0; base += 32) {
-          const int i = base + lane;
-          const unsigned m = __ballot_sync(FULL, i < r && __ldg(S.flavor + o + i) == f);
-          if (m) j = base + __ffs(m) - 1;
-        }
-        if (j < 0 || S.dagger[o + j] == S.dagger[o + r]) {
-          st = KT_EINVAL;
-        } else {
-          d = make_int4(1, r < j ? r : j, r < j ? j : r, K - 2);
-        }
-      }
-    } else {
-      st = KT_EINVAL;
-    }
-    if (st == KT_OK && cur_sign[w] == 0) st = KT_EZEROWEIGHT;
-  }
+  int4 d;
+  const int st = prep_walker(M, S, mv, has_moves, cur_sign, w, lane, d);
   if (lane == 0) {
     ws.desc[w] = d;
     ws.wstatus[w] = st;
@@ -566,6 +491,8 @@ int default_group_for(int kd, int precision) {
   return 32;
 }
 
+int default_eig_group_for(int kd) { return kd <= 10 ? 16 : 32; }
+
 int launch_pipeline(const DevModel &M, int precision, int kd, int G, const SeqView &S, const MoveView *moves,
                     const int8_t *cur_sign, const double *cur_logabs, int8_t *sign, double *logv, int32_t *status,
                     kt_stats *stats, const Workspace &ws, void *stream, const StageEvents *timing, double *obs) {
@@ -578,6 +505,16 @@ int launch_pipeline(const DevModel &M, int precision, int kd, int G, const SeqVi
   MoveView mv = moves ? *moves : MoveView{};
   cudaGetLastError();
   mark(0);
+  // Blocks of at most 36 rows: the whole call in the block eigenbasis, one kernel. Calls that
+  // count their work (stats) describe the Krylov propagation and therefore run it.
+  if (M.eig >= 0 && !stats) {
+    mark(1);
+    mark(2);
+    const int rc = launch_eig_pipeline(M, kd, G, S, moves, cur_sign, cur_logabs, sign, logv, status, ws, stream, obs);
+    mark(3);
+    mark(4);
+    return rc;
+  }
   prep_kernel<<<(n + 7) / 8, 256, 0, st>>>(M, S, mv, has_moves, cur_sign, ws, stats);
   mark(1);
   const long long items = (long long)n * M.n_kept;
@@ -607,6 +544,8 @@ int launch_cached_pipeline(const DevModel &M, int precision, int kd, const SeqVi
   cudaStream_t st = (cudaStream_t)stream;
   const int n = S.n;
   cudaGetLastError();
+  if (M.eig >= 0 && !stats)
+    return launch_eig_cached(M, kd, S, mv, cur_sign, cur_logabs, sign, logv, status, ws, C, write, stream);
   prep_kernel<<<(n + 7) / 8, 256, 0, st>>>(M, S, mv, 1, cur_sign, ws, stats);
   const long long items = (long long)n * M.n_kept;
   if (items > 0) {
@@ -629,6 +568,7 @@ int launch_cache_build(const DevModel &M, int precision, int kd, const SeqView &
   cudaStream_t st = (cudaStream_t)stream;
   const int n = S.n;
   cudaGetLastError();
+  if (M.eig >= 0) return launch_eig_build(M, kd, S, ws, C, stream);
   prep_kernel<<<(n + 7) / 8, 256, 0, st>>>(M, S, MoveView{}, 0, nullptr, ws, nullptr);
   const long long items = (long long)n * M.n_kept;
   if (items == 0) return (int)cudaGetLastError();
@@ -647,6 +587,7 @@ int launch_cached_measure(const DevModel &M, int precision, int kd, const SeqVie
   cudaStream_t st = (cudaStream_t)stream;
   const int n = S.n;
   cudaGetLastError();
+  if (M.eig >= 0) return launch_eig_measure(M, kd, S, sign, logv, status, obs, ws, C, stream);
   prep_kernel<<<(n + 7) / 8, 256, 0, st>>>(M, S, MoveView{}, 0, nullptr, ws, nullptr);
   const long long items = (long long)n * M.n_kept;
   if (items > 0) {

@@ -95,6 +95,7 @@ struct kt_model {
   kt::DevModel dev{};
   void *dev_mem = nullptr;
   size_t dev_bytes = 0;
+  void *eig_mem = nullptr;  // operator matrices between the block eigenbases
   int kernel_dmax = 0;
   int group_lanes = 32;
   int nnz_max = 0;
@@ -454,6 +455,27 @@ kt_status kt_model_create(const kt_model_params *pp, kt_model **out) {
       }
     }
 
+  // ---- block keys for the traces in the block eigenbasis: (n_up, n_dn, mask), followed through
+  //      a sequence as sums; an operator must reach a block exactly when the moved key has one ----
+  const int key_mask = sector_blocks ? 0 : (1 << n) - 1;
+  std::vector<int16_t> key_lut((size_t)((n + 1) * (n + 1)) << n, (int16_t)-1);
+  std::vector<int32_t> blk_key(B);
+  for (auto &kv : key2blk) {
+    const int nu = std::get<0>(kv.first), nd = std::get<1>(kv.first), mask = std::get<2>(kv.first);
+    blk_key[kv.second] = nu + 1024 * nd + (mask << 20);
+    key_lut[((size_t)(nu * (n + 1) + nd) << n) | mask] = (int16_t)kv.second;
+  }
+  bool keys_follow = true;
+  for (int b = 0; b < B; ++b)
+    for (int f = 0; f < nf; ++f)
+      for (int dg = 0; dg < 2; ++dg) {
+        const int s = dg ? 1 : -1, nu = (blk_key[b] & 1023) + (f & 1 ? 0 : s);
+        const int nd = ((blk_key[b] >> 10) & 1023) + (f & 1 ? s : 0), mask = (blk_key[b] >> 20) ^ ((1 << (f >> 1)) & key_mask);
+        const bool in = nu >= 0 && nu <= n && nd >= 0 && nd <= n;
+        const int t = in ? key_lut[((size_t)(nu * (n + 1) + nd) << n) | mask] : -1;
+        keys_follow = keys_follow && t == blk_target[((size_t)b * nf + f) * 2 + dg];
+      }
+
   // ---- spectrum, E0, kept multiplets ----
   struct Lv { double e; int b, j; };
   std::vector<Lv> lv;
@@ -474,11 +496,13 @@ kt_status kt_model_create(const kt_model_params *pp, kt_model **out) {
     i = j;
   }
   const int NK = (int)kept.size();
-  std::vector<int32_t> kept_blk(NK), kept_off(NK);
+  std::vector<int32_t> kept_blk(NK), kept_off(NK), kept_key(NK), kept_row(NK);
   std::vector<double> kept_e(NK), kept_vec64;
   for (int k = 0; k < NK; ++k) {
     const int b = kept[k].b, d = blk_dim[b];
     kept_blk[k] = b;
+    kept_key[k] = blk_key[b];
+    kept_row[k] = kept[k].j;
     kept_e[k] = kept[k].e - E0;
     kept_off[k] = (int32_t)kept_vec64.size();
     for (int r = 0; r < d; ++r) kept_vec64.push_back(evecs[b][(size_t)r * d + kept[k].j]);
@@ -530,6 +554,48 @@ kt_status kt_model_create(const kt_model_params *pp, kt_model **out) {
       }
     }
   }
+  // Traces in the block eigenbasis (kt_eig.cuh) for blocks of at most 36 rows, unless the caller
+  // lowered the Krylov cap below the block size: its KT_ENOCONV outcomes need the Krylov steps.
+  const int eig = !keys_follow || M->kernel_dmax > 36 || M->dev.pmax < std::min(d_max, kt::kernel_pmax_for(M->kernel_dmax))
+                      ? -1
+                      : P.precision == KT_FP64 ? 1 : 0;  // EIG_F64, EIG_PAIR
+  const int epv = 2;                 // matrix elements per 16-byte vector
+  std::vector<int32_t> eig_op;       // int4 entries
+  std::vector<double> eig_base(B), eig_lam64, eig_tab64, evec64;
+  std::vector<float> eig_lam32, eig_tab32;
+  size_t eig_vecs = 0;
+  if (eig >= 0) {
+    M->group_lanes = kt::default_eig_group_for(M->kernel_dmax);
+    eig_op.resize((size_t)B * nf * 2 * 4);
+    for (size_t i = 0; i < (size_t)B * nf * 2; ++i) {
+      const int b = (int)(i / (2 * nf)), t = blk_target[i];
+      eig_op[4 * i] = (int32_t)eig_vecs;
+      eig_op[4 * i + 1] = t < 0 ? 0 : blk_off[t] | blk_dim[b] << 16 | blk_dim[t] << 22;
+      eig_op[4 * i + 2] = t;
+      eig_op[4 * i + 3] = 0;
+      if (t >= 0) eig_vecs += (size_t)blk_dim[t] * ((blk_dim[b] + epv - 1) / epv);
+    }
+    const double log2e = 1.4426950408889634074;
+    for (int b = 0; b < B; ++b) {
+      eig_base[b] = blk_shift[b] - E0;
+      for (int k = 0; k < blk_dim[b]; ++k) {
+        const double l = st_eval64[blk_off[b] + k] * log2e;
+        if (eig == 1) {
+          eig_lam64.push_back(l);
+        } else {
+          eig_lam32.push_back((float)l);
+          eig_lam32.push_back((float)(l - (double)(float)l));
+        }
+        for (int r = 0; r < blk_dim[b]; ++r) evec64.push_back(evecs[b][(size_t)r * blk_dim[b] + k]);
+      }
+    }
+    for (int j = 0; eig == 1 && j < 128; ++j) eig_tab64.push_back(std::exp2(j / 128.0));
+    for (int j = 0; eig != 1 && j < 32; ++j) {
+      const double t = std::exp2(j / 32.0);
+      eig_tab32.push_back((float)t);
+      eig_tab32.push_back((float)(t - (double)(float)t));
+    }
+  }
   struct Piece { const void *src; size_t bytes; size_t off; };
   std::vector<Piece> pieces;
   size_t total = 0;
@@ -550,7 +616,13 @@ kt_status kt_model_create(const kt_model_params *pp, kt_model **out) {
                i_s2w = add(blk_s2w.data(), B * 4), i_s2o = add(blk_s2ell.data(), B * 4),
                i_sev64 = add(st_eval64.data(), N * 8), i_sev32 = add(st_eval32.data(), N * 4),
                i_evo = add(blk_evoff.data(), B * 4), i_evv = add(blk_evec32.data(), blk_evec32.size() * 4),
-               i_evvlo = add(blk_evec32lo.data(), blk_evec32lo.size() * 4);
+               i_evvlo = add(blk_evec32lo.data(), blk_evec32lo.size() * 4),
+               i_lut = add(key_lut.data(), key_lut.size() * 2), i_key = add(blk_key.data(), B * 4),
+               i_kk = add(kept_key.data(), NK * 4), i_kr = add(kept_row.data(), NK * 4),
+               i_eop = add(eig_op.data(), eig_op.size() * 4), i_eb = add(eig_base.data(), B * 8),
+               i_el = eig == 1 ? add(eig_lam64.data(), eig_lam64.size() * 8) : add(eig_lam32.data(), eig_lam32.size() * 4),
+               i_et = eig == 1 ? add(eig_tab64.data(), eig_tab64.size() * 8) : add(eig_tab32.data(), eig_tab32.size() * 4),
+               i_ev6 = add(evec64.data(), evec64.size() * 8);
   void *dmem = nullptr;
   if (cudaMalloc(&dmem, total) != cudaSuccess) { cudaGetLastError(); delete M; return KT_ENOMEM; }
   std::vector<char> host(total, 0);
@@ -589,6 +661,29 @@ kt_status kt_model_create(const kt_model_params *pp, kt_model **out) {
   D.blk_evec32lo = (const float *)at(i_evvlo);
   D.s2_diag = (const float *)at(i_s2d); D.s2_ell = (const uint16_t *)at(i_s2e);
   D.blk_s2w = (const int32_t *)at(i_s2w); D.blk_s2ell = (const int32_t *)at(i_s2o);
+  D.eig = eig;
+  D.key_mask = key_mask;
+  D.key_lut = (const int16_t *)at(i_lut); D.blk_key = (const int32_t *)at(i_key);
+  D.kept_key = (const int32_t *)at(i_kk); D.kept_row = (const int32_t *)at(i_kr);
+  D.eig_op = (const int4 *)at(i_eop); D.eig_base = (const double *)at(i_eb);
+  D.eig_lam = at(i_el); D.eig_tab = at(i_et); D.blk_evec64 = (const double *)at(i_ev6);
+  if (eig >= 0) {
+    const size_t bytes = std::max<size_t>(eig_vecs, 1) * 16;
+    if (cudaMalloc(&M->eig_mem, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      M->eig_mem = nullptr;
+      kt_model_destroy(M);
+      return KT_ENOMEM;
+    }
+    D.eig_mat = M->eig_mem;
+    M->dev_bytes += bytes;
+    // the caller may use the model on any stream at once: the matrices are complete on return
+    if (kt::build_eig_matrices(D) != 0 || cudaStreamSynchronize(0) != cudaSuccess) {
+      cudaGetLastError();
+      kt_model_destroy(M);
+      return KT_ECUDA;
+    }
+  }
   *out = M;
   return KT_OK;
 }
@@ -624,6 +719,7 @@ void kt_model_destroy(kt_model *m) {
   if (!m) return;
   timing_release(m);
   if (m->dev_mem) cudaFree(m->dev_mem);
+  if (m->eig_mem) cudaFree(m->eig_mem);
   delete m;
 }
 
