@@ -94,9 +94,124 @@ __device__ __forceinline__ void stage_tile(uint8_t *dst, const __nv_bfloat16 *sr
   }
 }
 
+// What a tile's epilogue makes of the accumulator. The network's layers apply their bias, ReLU, mask and
+// rounding here, on the values in registers: as kernels of their own over the FP32 matrices
+// (act1, dz1, gb1, transposes, 4,096 x 256 values each) they were 13 of a training step's 24 launches.
+//   EPI_STORE  C = acc
+//   EPI_ACT1   H1 = bf16(relu(acc + bias)), with C the FP32 acc too, with hT the transpose too
+//   EPI_OUT    y = v . relu(acc + bias) + *vb, for tiles that hold whole rows (N = 256 = BN)
+//   EPI_DZ1    C = acc (dH1), hT = transpose of bf16(acc masked by Z + bias > 0), part = column sums of
+//              the masked FP32 values per 32 rows
+enum { EPI_STORE, EPI_ACT1, EPI_OUT, EPI_DZ1 };
+struct Epi {
+  float *C;
+  int ldc;
+  const float *bias;
+  __nv_bfloat16 *h, *hT;  // [M][ldc], [N][M]
+  const float *Z;         // [M][ldc]
+  float *part;            // [ceil(M / 32)][ldc]
+  const float *v, *vb;
+  float *y;
+};
+
+// Warp w holds rows m0 + 32w .. (one per lane); 32 accumulator columns at a time. `tile`: 4 x 32 x 33
+// floats of shared memory (EPI_DZ1). A lane writes 16 bytes at a time where C allows it, transposes
+// are written by 32 consecutive rows.
+template <int EPI>
+__device__ __forceinline__ void tile_epilogue(uint32_t tmem, int m0, int n0, int bn, int M, const Epi &e, float *tile) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, row = m0 + warp * 32 + lane;
+  const bool vec = (e.ldc & 3) == 0 && ((uintptr_t)e.C & 15) == 0;
+  float acc[EPI == EPI_OUT ? 32 : 1];
+  if constexpr (EPI == EPI_OUT)
+#pragma unroll
+    for (int j = 0; j < 32; ++j) acc[j] = 0.f;
+  for (int c0 = 0; c0 < bn; c0 += 32) {
+    uint32_t r[32];
+    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    const int n = n0 + c0;
+    if (e.C && row < M) {
+      float *c = e.C + (size_t)row * e.ldc + n;
+      if (vec) {
+#pragma unroll
+        for (int j = 0; j < 32; j += 4)
+          if (c0 + j < bn)
+            *reinterpret_cast<float4 *>(c + j) = make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
+                                                             __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+      } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+          if (c0 + j < bn) c[j] = __uint_as_float(r[j]);
+      }
+    }
+    if constexpr (EPI == EPI_ACT1) {
+      if (row < M) {
+        uint32_t h[16];
+#pragma unroll
+        for (int j = 0; j < 32; j += 2) {
+          const __nv_bfloat16 a = __float2bfloat16_rn(fmaxf(__uint_as_float(r[j]) + __ldg(e.bias + n + j), 0.f));
+          const __nv_bfloat16 b = __float2bfloat16_rn(fmaxf(__uint_as_float(r[j + 1]) + __ldg(e.bias + n + j + 1), 0.f));
+          h[j / 2] = (uint32_t)__bfloat16_as_ushort(a) | (uint32_t)__bfloat16_as_ushort(b) << 16;
+          if (e.hT) {
+            e.hT[(size_t)(n + j) * M + row] = a;
+            e.hT[(size_t)(n + j + 1) * M + row] = b;
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          reinterpret_cast<uint4 *>(e.h + (size_t)row * e.ldc + n)[q] =
+              make_uint4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
+      }
+    } else if constexpr (EPI == EPI_OUT) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        acc[j] = fmaf(fmaxf(__uint_as_float(r[j]) + __ldg(e.bias + n + j), 0.f), __ldg(e.v + n + j), acc[j]);
+    } else if constexpr (EPI == EPI_DZ1) {
+      float *t = tile + warp * 32 * 33;
+      const float4 *z = reinterpret_cast<const float4 *>(e.Z + (size_t)row * e.ldc + n);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float4 zq = row < M ? z[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float zz[4] = {zq.x, zq.y, zq.z, zq.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int j = 4 * q + i;
+          const float d = row < M && zz[i] + __ldg(e.bias + n + j) > 0.f ? __uint_as_float(r[j]) : 0.f;
+          if (row < M) e.hT[(size_t)(n + j) * M + row] = __float2bfloat16_rn(d);
+          t[lane * 33 + j] = d;
+        }
+      }
+      __syncwarp();
+      float sum = 0.f;
+#pragma unroll 8
+      for (int i = 0; i < 32; ++i) sum += t[i * 33 + lane];
+      if (m0 + warp * 32 < M) e.part[(size_t)((m0 >> 5) + warp) * e.ldc + n + lane] = sum;
+      __syncwarp();
+    }
+  }
+  if constexpr (EPI == EPI_OUT) {
+    // the order of a warp's butterfly over 32 lanes
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int j = 0; j < o; ++j) acc[j] += acc[j + o];
+    if (row < M) e.y[row] = acc[0] + __ldg(e.vb);
+  }
+}
+
+template <int EPI>
 __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __nv_bfloat16 *__restrict__ A, int lda,
-                                                        const __nv_bfloat16 *__restrict__ B, int ldb, float *C, int ldc,
-                                                        int M, int N, int K, int BN, int kslice, int *err) {
+                                                        const __nv_bfloat16 *__restrict__ B, int ldb, Epi epi, int M,
+                                                        int N, int K, int BN, int kslice, int *err) {
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t *sA = smem;                      // 128 x 64 BF16 = 16 KB
   uint8_t *sB = smem + BM * BK * 2;        // BN x 64 BF16 <= 32 KB
@@ -109,7 +224,7 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __nv_bfloat16 *__r
   const int kb = blockIdx.z * kslice;
   A += kb;
   B += kb;
-  C += (size_t)blockIdx.z * M * ldc;
+  if (EPI == EPI_STORE) epi.C += (size_t)blockIdx.z * M * epi.ldc;
   K = min(K - kb, kslice);
   const int bn = (N - n0) < BN ? (N - n0) : BN;  // multiple of 16 (N is)
   const uint32_t ncols = 256;                    // power of two >= bn
@@ -168,29 +283,7 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __nv_bfloat16 *__r
     }
   }
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (!abort_sh) {
-    // epilogue: warp w reads TMEM lanes 32w .. 32w+31 (rows), 32 columns at a time
-    const int row = m0 + warp * 32 + lane;
-    for (int c0 = 0; c0 < bn; c0 += 32) {
-      uint32_t r[32];
-      const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-          "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-          "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-            "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-            "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-            "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-          : "r"(taddr));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (row < M) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (c0 + j < bn) C[(size_t)row * ldc + n0 + c0 + j] = __uint_as_float(r[j]);
-      }
-    }
-  }
+  if (!abort_sh) tile_epilogue<EPI>(tmem, m0, n0, bn, M, epi, reinterpret_cast<float *>(smem));
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
@@ -217,9 +310,10 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
       : "memory");
 }
 
+template <int EPI>
 __global__ void __launch_bounds__(128) gemm_bf16_tma_kernel(const __grid_constant__ CUtensorMap ta,
-                                                            const __grid_constant__ CUtensorMap tb, float *C, int ldc,
-                                                            int M, int N, int K, int BN, int kslice, int *err) {
+                                                            const __grid_constant__ CUtensorMap tb, Epi epi, int M,
+                                                            int N, int K, int BN, int kslice, int *err) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], done;
   __shared__ uint32_t tmem_base_sh;
@@ -231,7 +325,7 @@ __global__ void __launch_bounds__(128) gemm_bf16_tma_kernel(const __grid_constan
   const int bn = (N - n0) < BN ? (N - n0) : BN;
   const int kb = blockIdx.z * kslice, ke = min(K, kb + kslice);
   const int nchunks = (ke - kb + BK - 1) / BK;
-  C += (size_t)blockIdx.z * M * ldc;
+  if (EPI == EPI_STORE) epi.C += (size_t)blockIdx.z * M * epi.ldc;
   const uint32_t ncols = 256;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -306,28 +400,7 @@ __global__ void __launch_bounds__(128) gemm_bf16_tma_kernel(const __grid_constan
   __syncwarp();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   __syncthreads();
-  if (!abort_sh) {
-    const int row = m0 + warp * 32 + lane;
-    for (int c0 = 0; c0 < bn; c0 += 32) {
-      uint32_t r[32];
-      const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-          "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-          "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-            "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-            "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-            "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-          : "r"(taddr));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (row < M) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (c0 + j < bn) C[(size_t)row * ldc + n0 + c0 + j] = __uint_as_float(r[j]);
-      }
-    }
-  }
+  if (!abort_sh) tile_epilogue<EPI>(tmem, m0, n0, bn, M, epi, reinterpret_cast<float *>(smem));
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
@@ -356,18 +429,21 @@ int gemm_splits(int K, int splits) {
   return (K + kslice - 1) / kslice;
 }
 
-// C = A . B^T; requirements checked by the caller-facing entry point. The TMA-fed kernel
-// when the driver provides tensor maps, else the kernel that stages with ordinary loads.
-int gemm_bf16(const void *A, int lda, const void *B, int ldb, float *C, int ldc, int M, int N, int K, int *err,
-              void *st_, int splits) {
-  cudaStream_t st = (cudaStream_t)st_;
+// acc = A . B^T through a tile epilogue; requirements checked by the caller-facing entry points. The
+// TMA-fed kernel when the driver provides tensor maps, else the kernel that stages with ordinary loads.
+template <int EPI>
+int gemm_tiles(const void *A, int lda, const void *B, int ldb, const mlp::Epi &epi, int M, int N, int K, int *err,
+               cudaStream_t st, int splits = 1) {
   // column tile: the whole N when it fits the accumulator, narrower (128, then 64 columns)
   // while the grid would have fewer than 64 CTAs, so that small batches still spread out
   const int gm = (M + mlp::BM - 1) / mlp::BM, gz = gemm_splits(K, splits);
   int BN = N <= mlp::MAX_BN ? N : 128;
-  for (const int w : {128, 64})
-    if (BN > w && gm * ((N + BN - 1) / BN) * gz < 64) BN = w;
-  const int kslice_t = ((K + splits - 1) / splits + mlp::BK - 1) / mlp::BK * mlp::BK;
+  if (EPI != mlp::EPI_OUT)  // whole rows in one tile
+    for (const int w : {128, 64})
+      if (BN > w && gm * ((N + BN - 1) / BN) * gz < 64) BN = w;
+  // every slice holds at least one 64-column chunk of K (its offset keeps rows 16-byte aligned)
+  const int kslice = ((K + splits - 1) / splits + mlp::BK - 1) / mlp::BK * mlp::BK;
+  const dim3 grid((unsigned)gm, (unsigned)((N + BN - 1) / BN), (unsigned)((K + kslice - 1) / kslice));
   if (PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder()) {
     CUtensorMap ta, tb;
     const cuuint64_t da[2] = {(cuuint64_t)K, (cuuint64_t)M}, db[2] = {(cuuint64_t)K, (cuuint64_t)N};
@@ -382,26 +458,22 @@ int gemm_bf16(const void *A, int lda, const void *B, int ldb, float *C, int ldc,
       const size_t smem_t = (size_t)mlp::STAGES * ((size_t)mlp::BM * mlp::BK * 2 + (size_t)BN * mlp::BK * 2);
       static bool attr_t = false;
       if (!attr_t) {
-        cudaFuncSetAttribute(mlp::gemm_bf16_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(mlp::gemm_bf16_tma_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(mlp::STAGES * (mlp::BM + mlp::MAX_BN) * mlp::BK * 2));
         attr_t = true;
       }
-      dim3 grid((unsigned)gm, (unsigned)((N + BN - 1) / BN), (unsigned)((K + kslice_t - 1) / kslice_t));
-      mlp::gemm_bf16_tma_kernel<<<grid, 128, smem_t, st>>>(ta, tb, C, ldc, M, N, K, BN, kslice_t, err);
+      mlp::gemm_bf16_tma_kernel<EPI><<<grid, 128, smem_t, st>>>(ta, tb, epi, M, N, K, BN, kslice, err);
       return (int)cudaGetLastError();
     }
   }
   const size_t smem = (size_t)mlp::BM * mlp::BK * 2 + (size_t)BN * mlp::BK * 2;
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(mlp::gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+    cudaFuncSetAttribute(mlp::gemm_bf16_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
     attr = true;
   }
-  // every slice holds at least one 64-column chunk of K (its offset keeps rows 16-byte aligned)
-  const int kslice = ((K + splits - 1) / splits + mlp::BK - 1) / mlp::BK * mlp::BK;
-  dim3 grid((unsigned)((M + mlp::BM - 1) / mlp::BM), (unsigned)((N + BN - 1) / BN), (unsigned)((K + kslice - 1) / kslice));
-  mlp::gemm_bf16_kernel<<<grid, 128, smem, st>>>((const __nv_bfloat16 *)A, lda, (const __nv_bfloat16 *)B, ldb, C, ldc,
-                                                 M, N, K, BN, kslice, err);
+  mlp::gemm_bf16_kernel<EPI><<<grid, 128, smem, st>>>((const __nv_bfloat16 *)A, lda, (const __nv_bfloat16 *)B, ldb, epi,
+                                                      M, N, K, BN, kslice, err);
   return (int)cudaGetLastError();
 }
 
@@ -430,138 +502,198 @@ __global__ void transpose_bf16_kernel(const float *__restrict__ src, __nv_bfloat
   dst[(size_t)c * R + r] = __float2bfloat16_rn(src[i]);
 }
 
-// dst[c][r] = src[r][c] for BF16 matrices
-__global__ void transpose_b16_kernel(const __nv_bfloat16 *__restrict__ src, __nv_bfloat16 *dst, int R, int C) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)R * C) return;
-  const int r = (int)(i / C), c = (int)(i - (long long)r * C);
-  dst[(size_t)c * R + r] = src[i];
-}
-
-// H1 = relu(Z1 + b1) in BF16 (row-major; with HT also transposed)
-__global__ void act1_kernel(const float *__restrict__ Z1, const float *__restrict__ b1, __nv_bfloat16 *H1,
-                            __nv_bfloat16 *H1T, int B) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)B * H) return;
-  const int b = (int)(i / H), j = (int)(i - (long long)b * H);
-  const __nv_bfloat16 h = __float2bfloat16_rn(fmaxf(Z1[i] + b1[j], 0.f));
-  H1[i] = h;
-  if (H1T) H1T[(size_t)j * B + b] = h;
-}
-
-// y_b = w3 . relu(Z2_b + b2) + b3 (warp per row); H2 keeps relu(...) when given
-__global__ void out_kernel(const float *__restrict__ Z2, const float *__restrict__ b2, const float *__restrict__ w3,
-                           const float *__restrict__ b3, float *H2, float *y, int B) {
-  const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (row >= B) return;
-  float acc = 0.f;
-  for (int j = lane; j < H; j += 32) {
-    const float h = fmaxf(Z2[(size_t)row * H + j] + b2[j], 0.f);
-    if (H2) H2[(size_t)row * H + j] = h;
-    acc = fmaf(h, w3[j], acc);
+// Training, after z2: a block of 256 threads takes 32 rows (4 per warp, a lane every 32nd column) from
+// z2 to y, the loss, dy = 2 (y - t) / B and dZ2 = bf16(dy w3 masked by relu'(z2 + b2)) in both layouts,
+// and leaves its rows' sums of dy H2, of the unrounded dZ2 and of dy; Z2 is read once. The blocks from n_out
+// on transpose X in tiles of 64 x 64 for dW1, which has nothing to wait for. One launch for what were
+// six and a memset: every one of them ran 2 to 9 microseconds on a few megabytes from L2.
+constexpr int ROWS = 32, PITCH = ROWS + 2;
+struct OutTrain {
+  const float *Z2, *b2, *w3, *b3, *t;
+  float *y, *dy;
+  __nv_bfloat16 *dZ2, *dZ2T;
+  float *pw3, *pb2, *pb3, *ploss;  // per block of rows
+  const __nv_bfloat16 *X;
+  __nv_bfloat16 *XT;
+  int B, nin, n_out;
+};
+__global__ void __launch_bounds__(256) out_train_kernel(OutTrain A) {
+  __shared__ __align__(16) __nv_bfloat16 tile[H * PITCH];
+  __shared__ float sw3[8][H], sb2[8][H], sdy[8], slo[8];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, B = A.B;
+  if ((int)blockIdx.x >= A.n_out) {
+    constexpr int P = 66;
+    const int nk = (A.nin + 63) / 64, id = blockIdx.x - A.n_out, k0 = id % nk * 64, r0 = id / nk * 64;
+    for (int c = tid; c < 64 * 8; c += 256) {
+      const int r = c >> 3, k = (c & 7) * 8;
+      if (r0 + r >= B || k0 + k >= A.nin) continue;
+      const uint4 v = *reinterpret_cast<const uint4 *>(A.X + (size_t)(r0 + r) * A.nin + k0 + k);
+      uint32_t *d = reinterpret_cast<uint32_t *>(tile + r * P + k);
+      d[0] = v.x;
+      d[1] = v.y;
+      d[2] = v.z;
+      d[3] = v.w;
+    }
+    __syncthreads();
+    for (int c = tid; c < 64 * 8; c += 256) {
+      const int k = c >> 3, r = (c & 7) * 8;
+      if (k0 + k >= A.nin || r0 + r >= B) continue;
+      uint32_t v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        v[i] = (uint32_t)__bfloat16_as_ushort(tile[(r + 2 * i) * P + k]) |
+               (uint32_t)__bfloat16_as_ushort(tile[(r + 2 * i + 1) * P + k]) << 16;
+      *reinterpret_cast<uint4 *>(A.XT + (size_t)(k0 + k) * B + r0 + r) = make_uint4(v[0], v[1], v[2], v[3]);
+    }
+    return;
+  }
+  const int r0 = blockIdx.x * ROWS, rows = min(ROWS, B - r0);
+  float b2[8], w3[8], a[8], s[8], sd = 0.f, lo = 0.f;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    b2[k] = __ldg(A.b2 + lane + 32 * k);
+    w3[k] = __ldg(A.w3 + lane + 32 * k);
+    a[k] = s[k] = 0.f;
+  }
+  const float b3 = __ldg(A.b3);
+#pragma unroll
+  for (int i = 0; i < ROWS / 8; ++i) {
+    const int rr = warp * (ROWS / 8) + i, row = r0 + rr;
+    if (rr >= rows) break;
+    float z[8], acc = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      z[k] = A.Z2[(size_t)row * H + lane + 32 * k] + b2[k];
+      acc = fmaf(fmaxf(z[k], 0.f), w3[k], acc);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    const float y = acc + b3, e = y - A.t[row], d = 2.f * e / (float)B;
+    if (lane == 0) {
+      A.y[row] = y;
+      A.dy[row] = d;
+    }
+    sd += d;
+    lo += e * e / (float)B;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int j = lane + 32 * k;
+      const __nv_bfloat16 v = __float2bfloat16_rn(z[k] > 0.f ? d * w3[k] : 0.f);
+      A.dZ2[(size_t)row * H + j] = v;
+      tile[j * PITCH + rr] = v;
+      a[k] = fmaf(d, fmaxf(z[k], 0.f), a[k]);
+      if (z[k] > 0.f) s[k] = fmaf(d, w3[k], s[k]);
+    }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) y[row] = acc + b3[0];
-}
-
-// dy = 2 (y - t) / B; loss += (y - t)^2 / B
-__global__ void loss_kernel(const float *__restrict__ y, const float *__restrict__ t, float *dy, float *loss, int B) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  float c = 0.f;
-  if (b < B) {
-    const float r = y[b] - t[b];
-    dy[b] = 2.f * r / (float)B;
-    c = r * r / (float)B;
+  for (int k = 0; k < 8; ++k) {
+    sw3[warp][lane + 32 * k] = a[k];
+    sb2[warp][lane + 32 * k] = s[k];
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if ((threadIdx.x & 31) == 0 && c != 0.f) atomicAdd(loss, c);
-}
-
-// dZ2 = dy w3^T masked by relu'(Z2 + b2), BF16 in both layouts
-__global__ void dz2_kernel(const float *__restrict__ Z2, const float *__restrict__ b2, const float *__restrict__ w3,
-                           const float *__restrict__ dy, __nv_bfloat16 *dZ2, __nv_bfloat16 *dZ2T, int B) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)B * H) return;
-  const int b = (int)(i / H), j = (int)(i - (long long)b * H);
-  const float d = (Z2[i] + b2[j] > 0.f) ? dy[b] * w3[j] : 0.f;
-  const __nv_bfloat16 v = __float2bfloat16_rn(d);
-  dZ2[i] = v;
-  dZ2T[(size_t)j * B + b] = v;
-}
-
-// Column sums over the batch, gw3_j = sum_b dy_b H2_bj, gb2_j = sum_b dZ2_bj and
-// gb3 = sum_b dy_b (FP32), in two deterministic passes: one block of H threads per chunk
-// of ROWS rows writes the chunk's sums, then one block adds the chunks in order.
-constexpr int ROWS = 128;
-__global__ void out_grads_part_kernel(const float *__restrict__ Z2, const float *__restrict__ b2,
-                                      const float *__restrict__ w3, const float *__restrict__ H2,
-                                      const float *__restrict__ dy, float *pw3, float *pb2, float *pb3, int B) {
-  __shared__ float sh[H];
-  const int c = blockIdx.x, j = threadIdx.x;
-  const int r0 = c * ROWS, r1 = min(B, r0 + ROWS);
-  float a = 0.f, s = 0.f;
-  for (int b = r0; b < r1; ++b) {
-    const float d = dy[b];
-    a = fmaf(d, H2[(size_t)b * H + j], a);
-    if (Z2[(size_t)b * H + j] + b2[j] > 0.f) s = fmaf(d, w3[j], s);
+  if (lane == 0) {
+    sdy[warp] = sd;
+    slo[warp] = lo;
   }
-  pw3[(size_t)c * H + j] = a;
-  pb2[(size_t)c * H + j] = s;
-  sh[j] = (j < ROWS && r0 + j < r1) ? dy[r0 + j] : 0.f;
   __syncthreads();
-  for (int o = H / 2; o > 0; o >>= 1) {
-    if (j < o) sh[j] += sh[j + o];
+  float x = 0.f, u = 0.f;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    x += sw3[q][tid];
+    u += sb2[q][tid];
+  }
+  A.pw3[(size_t)blockIdx.x * H + tid] = x;
+  A.pb2[(size_t)blockIdx.x * H + tid] = u;
+  if (tid == 0) {
+    float p = 0.f, l = 0.f;
+    for (int q = 0; q < 8; ++q) {
+      p += sdy[q];
+      l += slo[q];
+    }
+    A.pb3[blockIdx.x] = p;
+    A.ploss[blockIdx.x] = l;
+  }
+  // the transpose: 16 bytes (8 rows) per lane, four lanes per column
+  for (int c = tid; c < H * 4; c += 256) {
+    const int j = c >> 2, r = (c & 3) * 8;
+    if (r >= rows) continue;
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(tile + j * PITCH + r);
+    *reinterpret_cast<uint4 *>(A.dZ2T + (size_t)j * B + r0 + r) = make_uint4(src[0], src[1], src[2], src[3]);
+  }
+}
+
+// The gradients from their parts, one launch: the weight gradients' split-K slabs (in order), the
+// column sums of the blocks of rows (32 columns per block, 8 threads a column), db3 and the loss.
+struct Grads {
+  const float *part1, *part2;       // [S][H][nin], [S][H][H]
+  float *gW1, *gW2;
+  const float *pcol[3];             // dy H2, dZ2, dZ1: [nc][H]
+  float *gcol[3];                   // gw3, gb2, gb1
+  const float *pb3, *ploss;
+  float *gb3, *loss, *loss_out;
+  int S, nc, nin;
+};
+__global__ void __launch_bounds__(256) grads_kernel(Grads G, int n1, int n2) {
+  __shared__ float sh[2][256];
+  const int tid = threadIdx.x, blk = blockIdx.x;
+  if (blk < n1 + n2) {
+    const bool first = blk < n1;
+    const int i = ((first ? blk : blk - n1) * 256 + tid) * 4, n = H * (first ? G.nin : H);
+    if (i >= n) return;
+    const float *p = (first ? G.part1 : G.part2) + i;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int q = 0; q < G.S; ++q) {
+      const float4 v = *reinterpret_cast<const float4 *>(p + (size_t)q * n);
+      a.x += v.x;
+      a.y += v.y;
+      a.z += v.z;
+      a.w += v.w;
+    }
+    float *o = (first ? G.gW1 : G.gW2) + i;
+    *reinterpret_cast<float4 *>(o) = a;
+    return;
+  }
+  const int c = blk - n1 - n2;
+  if (c < 3 * H / 32) {
+    const int k = c / (H / 32), j = c % (H / 32) * 32 + (tid & 31);
+    const float *p = k == 0 ? G.pcol[0] : (k == 1 ? G.pcol[1] : G.pcol[2]);
+    float s = 0.f;
+    for (int q = tid >> 5; q < G.nc; q += 8) s += p[(size_t)q * H + j];
+    sh[0][tid] = s;
+    __syncthreads();
+    if (tid < 32) {
+      for (int q = 1; q < 8; ++q) s += sh[0][tid + 32 * q];
+      (k == 0 ? G.gcol[0] : (k == 1 ? G.gcol[1] : G.gcol[2]))[j] = s;
+    }
+    return;
+  }
+  float a = 0.f, b = 0.f;
+  for (int q = tid; q < G.nc; q += 256) {
+    a += G.pb3[q];
+    b += G.ploss[q];
+  }
+  sh[0][tid] = a;
+  sh[1][tid] = b;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (tid < o) {
+      sh[0][tid] += sh[0][tid + o];
+      sh[1][tid] += sh[1][tid + o];
+    }
     __syncthreads();
   }
-  if (j == 0) pb3[c] = sh[0];
-}
-__global__ void out_grads_sum_kernel(const float *__restrict__ pw3, const float *__restrict__ pb2,
-                                     const float *__restrict__ pb3, float *gw3, float *gb2, float *gb3, int nc) {
-  const int j = threadIdx.x;
-  float a = 0.f, s = 0.f, t = 0.f;
-  for (int c = 0; c < nc; ++c) {
-    a += pw3[(size_t)c * H + j];
-    s += pb2[(size_t)c * H + j];
-    if (j == 0) t += pb3[c];
+  if (tid == 0) {
+    G.gb3[0] = sh[0][0];
+    G.loss[0] = sh[1][0];
+    if (G.loss_out) G.loss_out[0] = sh[1][0];
   }
-  gw3[j] = a;
-  gb2[j] = s;
-  if (j == 0) gb3[0] = t;
 }
 
-// Sum of split-K partial products: out[i] = sum over slabs s of part[s n + i], in order.
-__global__ void splitk_sum_kernel(const float *__restrict__ part, float *out, int S, long long n) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float a = 0.f;
-  for (int s = 0; s < S; ++s) a += part[(size_t)s * n + i];
-  out[i] = a;
-}
-
-// dZ1 = dH1 masked by relu'(Z1 + b1): BF16 transposed [H][B]; gb1 column sums (FP32)
-__global__ void dz1_kernel(const float *__restrict__ dH1, const float *__restrict__ Z1, const float *__restrict__ b1,
-                           __nv_bfloat16 *dZ1T, int B) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)B * H) return;
-  const int b = (int)(i / H), j = (int)(i - (long long)b * H);
-  const float d = (Z1[i] + b1[j] > 0.f) ? dH1[i] : 0.f;
-  dZ1T[(size_t)j * B + b] = __float2bfloat16_rn(d);
-}
-__global__ void gb1_part_kernel(const float *__restrict__ dH1, const float *__restrict__ Z1,
-                                const float *__restrict__ b1, float *pb1, int B) {
-  const int c = blockIdx.x, j = threadIdx.x;
-  const int r0 = c * ROWS, r1 = min(B, r0 + ROWS);
-  float s = 0.f;
-  for (int b = r0; b < r1; ++b)
-    if (Z1[(size_t)b * H + j] + b1[j] > 0.f) s += dH1[(size_t)b * H + j];
-  pb1[(size_t)c * H + j] = s;
-}
-
-// Adam (Kingma & Ba 2015, Algorithm 1) on the packed FP32 parameters
+// Adam (Kingma & Ba 2015, Algorithm 1) on the packed FP32 parameters, and the BF16 operands made of W1
+// (at 0) and W2 (at o2; its transpose too)
 __global__ void adam_kernel(float *p, const float *__restrict__ g, float *m, float *v, long long n, float lr, float bc1,
-                            float bc2) {
+                            float bc2, __nv_bfloat16 *W1b, long long n1, __nv_bfloat16 *W2b, __nv_bfloat16 *W2Tb,
+                            long long o2) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float gi = g[i];
@@ -569,7 +701,16 @@ __global__ void adam_kernel(float *p, const float *__restrict__ g, float *m, flo
   const float vi = 0.999f * v[i] + 0.001f * gi * gi;
   m[i] = mi;
   v[i] = vi;
-  p[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + 1e-8f);
+  const float x = p[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + 1e-8f);
+  p[i] = x;
+  const __nv_bfloat16 b = __float2bfloat16_rn(x);
+  if (i < n1) {
+    W1b[i] = b;
+  } else if (i >= o2 && i < o2 + H * H) {
+    const int e = (int)(i - o2);
+    W2b[e] = b;
+    W2Tb[(e % H) * H + e / H] = b;
+  }
 }
 
 inline unsigned blocks(long long n, int t = 256) { return (unsigned)((n + t - 1) / t); }
@@ -585,10 +726,10 @@ struct kt_mlp {
   float *W1, *b1, *W2, *b2, *w3, *b3;
   float *gW1, *gb1, *gW2, *gb2, *gw3, *gb3;
   __nv_bfloat16 *W1b, *W2b, *W2Tb;
-  float *Z1, *Z2, *H2, *dH1, *y, *dy, *loss;
+  float *Z1, *Z2, *dH1, *y, *dy, *loss;
   __nv_bfloat16 *H1b, *H1Tb, *dZ2b, *dZ2Tb, *dZ1Tb, *XTb;
-  float *part;               // split-K slabs of the weight gradients
-  float *pw3, *pb2, *pb3, *pb1;  // per-chunk column sums
+  float *part1, *part2;      // split-K slabs of the weight gradients
+  float *pw3, *pb2, *pb3, *pb1, *ploss;  // sums of 32 rows
   int *err;
 };
 
@@ -605,17 +746,25 @@ int mlp_refresh_bf16(kt_mlp *n, cudaStream_t st) {
   return (int)cudaGetLastError();
 }
 
-// y[B] = network(X [B][n_in] BF16); with train, keeps what the backward pass needs
+// y[B] = network(X [B][n_in] BF16), two launches; with train, z1, H1 and its transpose and z2 for the
+// backward pass instead of y
 int mlp_forward(kt_mlp *n, const void *X, int B, float *y, bool train, void *st_) {
   using namespace mlp;
   cudaStream_t st = (cudaStream_t)st_;
-  int rc = gemm_bf16(X, n->n_in, n->W1b, n->n_in, n->Z1, H, B, H, n->n_in, n->err, st);
+  Epi e1{train ? n->Z1 : nullptr, H, n->b1, n->H1b, train ? n->H1Tb : nullptr};
+  const int rc = gemm_tiles<EPI_ACT1>(X, n->n_in, n->W1b, n->n_in, e1, B, H, n->n_in, n->err, st);
   if (rc) return rc;
-  act1_kernel<<<blocks((long long)B * H), 256, 0, st>>>(n->Z1, n->b1, n->H1b, train ? n->H1Tb : nullptr, B);
-  rc = gemm_bf16(n->H1b, H, n->W2b, H, n->Z2, H, B, H, H, n->err, st);
-  if (rc) return rc;
-  out_kernel<<<blocks((long long)B * 32), 256, 0, st>>>(n->Z2, n->b2, n->w3, n->b3, train ? n->H2 : nullptr, y, B);
-  return (int)cudaGetLastError();
+  Epi e2{};
+  e2.ldc = H;
+  if (train) {
+    e2.C = n->Z2;
+    return gemm_tiles<EPI_STORE>(n->H1b, H, n->W2b, H, e2, B, H, H, n->err, st);
+  }
+  e2.bias = n->b2;
+  e2.v = n->w3;
+  e2.vb = n->b3;
+  e2.y = y;
+  return gemm_tiles<EPI_OUT>(n->H1b, H, n->W2b, H, e2, B, H, H, n->err, st);
 }
 
 }  // namespace kt
@@ -640,11 +789,12 @@ kt_status kt_mlp_create(int32_t n_in, int32_t max_batch, kt_mlp **out) {
   };
   const size_t o_p = take(P * 4), o_g = take(P * 4), o_m = take(P * 4), o_v = take(P * 4),
                o_w1b = take((size_t)H * n_in * 2), o_w2b = take((size_t)H * H * 2), o_w2t = take((size_t)H * H * 2),
-               o_z1 = take(B * H * 4), o_z2 = take(B * H * 4), o_h2 = take(B * H * 4), o_dh1 = take(B * H * 4),
+               o_z1 = take(B * H * 4), o_z2 = take(B * H * 4), o_dh1 = take(B * H * 4),
                o_y = take(B * 4), o_dy = take(B * 4), o_loss = take(4), o_h1 = take(B * H * 2), o_h1t = take(B * H * 2),
                o_dz2 = take(B * H * 2), o_dz2t = take(B * H * 2), o_dz1t = take(B * H * 2),
                o_xt = take(B * (size_t)n_in * 2), o_err = take(4),
-               o_part = take((size_t)kt::mlp::MAX_SPLITS * H * (n_in > H ? n_in : H) * 4),
+               o_part1 = take((size_t)kt::mlp::MAX_SPLITS * H * n_in * 4),
+               o_part2 = take((size_t)kt::mlp::MAX_SPLITS * H * H * 4), o_ploss = take((B / ROWS + 1) * 4),
                o_pw3 = take((B / ROWS + 1) * H * 4), o_pb2 = take((B / ROWS + 1) * H * 4), o_pb3 = take((B / ROWS + 1) * 4),
                o_pb1 = take((B / ROWS + 1) * H * 4);
   if (cudaMalloc(&n->mem, off) != cudaSuccess) {
@@ -665,7 +815,9 @@ kt_status kt_mlp_create(int32_t n_in, int32_t max_batch, kt_mlp **out) {
   n->b2 = q; n->gb2 = r; q += H; r += H;
   n->w3 = q; n->gw3 = r; q += H; r += H;
   n->b3 = q; n->gb3 = r;
-  n->part = (float *)(b + o_part);
+  n->part1 = (float *)(b + o_part1);
+  n->part2 = (float *)(b + o_part2);
+  n->ploss = (float *)(b + o_ploss);
   n->pw3 = (float *)(b + o_pw3);
   n->pb2 = (float *)(b + o_pb2);
   n->pb3 = (float *)(b + o_pb3);
@@ -675,7 +827,6 @@ kt_status kt_mlp_create(int32_t n_in, int32_t max_batch, kt_mlp **out) {
   n->W2Tb = (__nv_bfloat16 *)(b + o_w2t);
   n->Z1 = (float *)(b + o_z1);
   n->Z2 = (float *)(b + o_z2);
-  n->H2 = (float *)(b + o_h2);
   n->dH1 = (float *)(b + o_dh1);
   n->y = (float *)(b + o_y);
   n->dy = (float *)(b + o_dy);
@@ -732,28 +883,24 @@ kt_status kt_mlp_backward(kt_mlp *n, const void *X, const float *t, int32_t B, f
   if (!n || !X || !t || B < 16 || (B % 16) || B > n->maxB || ((uintptr_t)X % 16)) return KT_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   const int nin = n->n_in;
-  if (kt::mlp_forward(n, X, B, n->y, true, st) != 0) return KT_ECUDA;
-  cudaMemsetAsync(n->loss, 0, 4, st);
-  loss_kernel<<<blocks(B), 256, 0, st>>>(n->y, t, n->dy, n->loss, B);
-  dz2_kernel<<<blocks((long long)B * H), 256, 0, st>>>(n->Z2, n->b2, n->w3, n->dy, n->dZ2b, n->dZ2Tb, B);
-  const int nc = (B + ROWS - 1) / ROWS;
-  out_grads_part_kernel<<<nc, H, 0, st>>>(n->Z2, n->b2, n->w3, n->H2, n->dy, n->pw3, n->pb2, n->pb3, B);
-  out_grads_sum_kernel<<<1, H, 0, st>>>(n->pw3, n->pb2, n->pb3, n->gw3, n->gb2, n->gb3, nc);
-  // weight gradients reduce over the batch: split K = B over several CTAs, then sum the slabs
-  const int S = kt::gemm_splits(B, MAX_SPLITS);
+  if (kt::mlp_forward(n, X, B, nullptr, true, st) != 0) return KT_ECUDA;
+  const int nc = (B + ROWS - 1) / ROWS, nt = (B + 63) / 64 * ((nin + 63) / 64);
+  out_train_kernel<<<nc + nt, 256, 0, st>>>(OutTrain{n->Z2, n->b2, n->w3, n->b3, t, n->y, n->dy, n->dZ2b, n->dZ2Tb, n->pw3,
+                                                     n->pb2, n->pb3, n->ploss, (const __nv_bfloat16 *)X, n->XTb, B, nin, nc});
+  // dH1 = dZ2 W2: A = dZ2 [B][H], B-operand = W2T [H(in)][H(out)]; its mask, dZ1 and db1 in the epilogue
+  Epi ed{n->dH1, H, n->b1, nullptr, n->dZ1Tb, n->Z1, n->pb1};
+  if (kt::gemm_tiles<EPI_DZ1>(n->dZ2b, H, n->W2Tb, H, ed, B, H, H, n->err, st)) return KT_ECUDA;
+  // weight gradients reduce over the batch: split K = B over several CTAs, the slabs summed below
   // dW2 = dZ2^T H1: A = dZ2T [H][B], B-operand = H1T [H][B]
-  if (kt::gemm_bf16(n->dZ2Tb, B, n->H1Tb, B, n->part, H, H, H, B, n->err, st, MAX_SPLITS)) return KT_ECUDA;
-  splitk_sum_kernel<<<blocks((long long)H * H), 256, 0, st>>>(n->part, n->gW2, S, (long long)H * H);
-  // dH1 = dZ2 W2: A = dZ2 [B][H], B-operand = W2T [H(in)][H(out)]
-  if (kt::gemm_bf16(n->dZ2b, H, n->W2Tb, H, n->dH1, H, B, H, H, n->err, st)) return KT_ECUDA;
-  dz1_kernel<<<blocks((long long)B * H), 256, 0, st>>>(n->dH1, n->Z1, n->b1, n->dZ1Tb, B);
-  gb1_part_kernel<<<nc, H, 0, st>>>(n->dH1, n->Z1, n->b1, n->pb1, B);
-  splitk_sum_kernel<<<1, H, 0, st>>>(n->pb1, n->gb1, nc, H);
+  Epi e2{n->part2, H};
+  if (kt::gemm_tiles<EPI_STORE>(n->dZ2Tb, B, n->H1Tb, B, e2, H, H, B, n->err, st, MAX_SPLITS)) return KT_ECUDA;
   // dW1 = dZ1^T X: A = dZ1T [H][B], B-operand = XT [n_in][B]
-  transpose_b16_kernel<<<blocks((long long)B * nin), 256, 0, st>>>((const __nv_bfloat16 *)X, n->XTb, B, nin);
-  if (kt::gemm_bf16(n->dZ1Tb, B, n->XTb, B, n->part, nin, H, nin, B, n->err, st, MAX_SPLITS)) return KT_ECUDA;
-  splitk_sum_kernel<<<blocks((long long)H * nin), 256, 0, st>>>(n->part, n->gW1, S, (long long)H * nin);
-  if (loss) cudaMemcpyAsync(loss, n->loss, 4, cudaMemcpyDeviceToDevice, st);
+  Epi e1{n->part1, nin};
+  if (kt::gemm_tiles<EPI_STORE>(n->dZ1Tb, B, n->XTb, B, e1, H, nin, B, n->err, st, MAX_SPLITS)) return KT_ECUDA;
+  const int n1 = (int)blocks((long long)H * nin / 4), n2 = (int)blocks((long long)H * H / 4);
+  grads_kernel<<<n1 + n2 + 3 * H / 32 + 1, 256, 0, st>>>(
+      Grads{n->part1, n->part2, n->gW1, n->gW2, {n->pw3, n->pb2, n->pb1}, {n->gw3, n->gb2, n->gb1}, n->pb3, n->ploss,
+            n->gb3, n->loss, loss, kt::gemm_splits(B, MAX_SPLITS), nc, nin}, n1, n2);
   n->lastB = B;
   return cudaGetLastError() == cudaSuccess ? KT_OK : KT_ECUDA;
 }
@@ -781,8 +928,8 @@ kt_status kt_mlp_adam(kt_mlp *n, float lr, void *stream) {
   cudaStream_t st = (cudaStream_t)stream;
   n->step += 1;
   const float bc1 = 1.f - powf(0.9f, (float)n->step), bc2 = 1.f - powf(0.999f, (float)n->step);
-  adam_kernel<<<blocks(n->P), 256, 0, st>>>(n->p, n->g, n->m, n->v, n->P, lr, bc1, bc2);
-  if (kt::mlp_refresh_bf16(n, st) != 0) return KT_ECUDA;
+  adam_kernel<<<blocks(n->P), 256, 0, st>>>(n->p, n->g, n->m, n->v, n->P, lr, bc1, bc2, n->W1b, (long long)H * n->n_in,
+                                            n->W2b, n->W2Tb, n->W2 - n->p);
   return cudaGetLastError() == cudaSuccess ? KT_OK : KT_ECUDA;
 }
 
@@ -805,5 +952,6 @@ extern "C" kt_status kt_gemm_bf16(const void *A, int32_t lda, const void *B, int
   if (!A || !B || !C || !err || M < 1 || N < 16 || K < 16 || (N % 16) || (K % 16) || lda < K || ldb < K || ldc < N ||
       (lda % 8) || (ldb % 8) || ((uintptr_t)A % 16) || ((uintptr_t)B % 16))
     return KT_EINVAL;
-  return kt::gemm_bf16(A, lda, B, ldb, C, ldc, M, N, K, err, stream) == 0 ? KT_OK : KT_ECUDA;
+  const kt::mlp::Epi epi{C, ldc};
+  return kt::gemm_tiles<kt::mlp::EPI_STORE>(A, lda, B, ldb, epi, M, N, K, err, (cudaStream_t)stream) == 0 ? KT_OK : KT_ECUDA;
 }
