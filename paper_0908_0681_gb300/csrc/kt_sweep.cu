@@ -118,30 +118,39 @@ __device__ __forceinline__ double hyb_F(const SweepView &S, int f, double t) {
   return a + fr * (b - a);
 }
 __device__ __forceinline__ double hyb_Fh(const SweepView &S, int f, double x) {
-  return x >= 0.0 ? hyb_F(S, f, x) : -hyb_F(S, f, x + S.beta);
+  const double v = hyb_F(S, f, x >= 0.0 ? x : x + S.beta);  // one evaluation for both signs of the lanes
+  return x >= 0.0 ? v : -v;
 }
+
+// A time (>= 0) as an integer of the same order: comparisons of times leave the FP64 pipe, which
+// issues one warp instruction per 16 cycles and SM.
+__device__ __forceinline__ long long time_key(double t) { return __double_as_longlong(t) & 0x7fffffffffffffffll; }
 
 __device__ __forceinline__ int warp_sum(int v) { return __reduce_add_sync(FULL, (unsigned)v); }
-__device__ __forceinline__ double warp_sum(double v) {
+// Indices of the operators number m[0], m[1], m[2] (0-based) of flavor f among ops[0 .. K), -1 where
+// there are fewer. Four chunks of 32 operators are loaded at a time.
+__device__ void three_of_flavor(const uint8_t *fl, int K, int f, const int (&m)[3], int (&at)[3], int lane) {
+  int cnt = 0, left = 3;
+  for (int r = 0; r < 3; ++r) at[r] = -1;
+  for (int base = 0; base < K && left > 0; base += 128) {
+    int g[4];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-  return v;
-}
-
-// Index of the m-th (0-based) operator of flavor f among ops[0 .. K), or -1.
-__device__ int nth_of_flavor(const uint8_t *fl, int K, int f, int m, int lane) {
-  int cnt = 0;
-  for (int base = 0; base < K; base += 32) {
-    const int idx = base + lane;
-    unsigned msk = __ballot_sync(FULL, idx < K && fl[idx] == f);
-    const int c = __popc(msk);
-    if (cnt + c > m) {
-      for (int r = m - cnt; r > 0; --r) msk &= msk - 1;
-      return base + __ffs(msk) - 1;
+    for (int c = 0; c < 4; ++c) g[c] = base + 32 * c + lane < K ? fl[base + 32 * c + lane] : 256;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const unsigned msk = __ballot_sync(FULL, g[c] == f);
+      const int n = __popc(msk);
+#pragma unroll
+      for (int r = 0; r < 3; ++r)
+        if (m[r] >= cnt && m[r] < cnt + n) {
+          unsigned x = msk;
+          for (int k = m[r] - cnt; k > 0; --k) x &= x - 1;
+          at[r] = base + 32 * c + __ffs(x) - 1;
+          --left;
+        }
+      cnt += n;
     }
-    cnt += c;
   }
-  return -1;
 }
 
 // Parity count X of the permutation sign change for a pair (tdag, tann) of flavor f
@@ -149,12 +158,13 @@ __device__ int nth_of_flavor(const uint8_t *fl, int K, int f, int m, int lane) {
 __device__ int perm_count(const double *tau, const uint8_t *fl, int K, int f, double tdag, double tann, int skip1,
                           int skip2, int lane) {
   int c = 0;
+  const long long kd = time_key(tdag), ka = time_key(tann);
+#pragma unroll 4
   for (int idx = lane; idx < K; idx += 32) {
-    if (idx == skip1 || idx == skip2) continue;
-    const double t = tau[idx];
+    const long long t = time_key(tau[idx]);
     const int g = fl[idx];
-    if (g <= f) c += (t < tdag) + (t < tann);
-    else c += (t > tdag) + (t > tann);
+    const int below = (t < kd) + (t < ka), above = (t > kd) + (t > ka);
+    c += idx == skip1 || idx == skip2 ? 0 : (g <= f ? below : above);
   }
   c = warp_sum(c);
   return c + (tdag < tann ? 1 : 0);
@@ -170,9 +180,12 @@ struct TryView {
   uint8_t *mv_kind, *mv_flv;
   __nv_bfloat16 *X;
   float *ytil;
-  unsigned long long *scratch_counters;  // the propose kernel's counters land here; the select kernel counts
   int32_t *n_tries;   // [nw] Metropolis steps the walker took this step (tries up to and including the selected one)
-  int16_t *nxt;       // [nw][cap] next operator of the same flavor (sweep_next_flavor_kernel)
+  // the configuration's segments (sweep_segments_kernel)
+  int16_t *nxt;       // [nw][cap] next operator of the same flavor, cyclically (-1: none)
+  double2 *seg_t;     // [nw][cap / 2] one segment per creator: its time and its end, time + length
+  uint2 *seg_m;       // [nw][cap / 2] creator | its next operator << 16, flavor | length bin << 8 (255: no segment)
+  int32_t *n_seg;     // [nw]
   double *u5;         // [nw] stage-2 uniform of the selected try
 };
 
@@ -186,11 +199,15 @@ __host__ __device__ inline SweepView try_view(const SweepView &S, const TryView 
   v.p_vec = Tv.p_vec + o * 2 * S.kcap; v.p_pair = Tv.p_pair + 2 * o; v.mv_rem = Tv.mv_rem + o;
   v.p_ij = Tv.p_ij + 2 * o; v.mv_kind = Tv.mv_kind + o; v.mv_flv = Tv.mv_flv + o;
   v.X = Tv.X + o * S.n_in; v.ytil = Tv.ytil + o;
-  v.counters = Tv.scratch_counters;
   return v;
 }
 
-// Tv.T > 0: multi-try launch, blockIdx.y = try (uniforms of try t at uni + 7 t).
+// Tv.T > 0: multi-try launch, blockIdx.y = try (uniforms of try t at uni + 7 t; the select kernel
+// counts the moves). The FP64 pipe bounds it: one warp instruction per 16 cycles and SM, where a log
+// is about 35 and a hybridization value, with its division, about 25. So the kf values of the new
+// column, the kf of the new row and the corner share one evaluation over the lanes, so do the two
+// matrix-vector products and the two logarithms, and times are compared as integers. 8,192 proposals
+// (1,024 chains at beta = 50, eight tries): 101 -> 54 us.
 __global__ void sweep_propose_kernel(SweepView S0, const double *__restrict__ uni, int ustride, TryView Tv) {
   extern __shared__ double sh[];
   const SweepView S = Tv.T ? try_view(S0, Tv, blockIdx.y) : S0;
@@ -198,8 +215,7 @@ __global__ void sweep_propose_kernel(SweepView S0, const double *__restrict__ un
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int w = blockIdx.x * (blockDim.x >> 5) + wib;
   if (w >= S.nw) return;
-  double *Cv = sh + (size_t)wib * 2 * S.kcap;  // new column C (by creator) / row R (by annihilator)
-  double *Rv = Cv + S.kcap;
+  double *CR = sh + (size_t)wib * (2 * S.kcap + 1);  // new column C (by creator), row R (by annihilator), corner
   const double *u = uni + (size_t)w * ustride;
   const int nf = S.nf;
   const double beta = S.beta;
@@ -224,25 +240,34 @@ __global__ void sweep_propose_kernel(SweepView S0, const double *__restrict__ un
   int valid = 0;
   if (u[0] < 0.5) {
     // ---- insertion ----
-    if (lane == 0) atomicAdd(&S.counters[C_INS_PROP], 1ull);
+    if (lane == 0 && !Tv.T) atomicAdd(&S.counters[C_INS_PROP], 1ull);
     const double t1 = u[2] * beta;
     bool null_move = false;
     if (kf >= S.kcap) {
       null_move = true;
-      if (lane == 0) atomicAdd(&S.counters[C_CAP], 1ull);
+      if (lane == 0 && !Tv.T) atomicAdd(&S.counters[C_CAP], 1ull);
     }
     if (!(t1 < beta)) null_move = true;
     bool seg = true;
     double lmax = beta;
     if (!null_move && kf > 0) {
       int first_any = -1, found = -1;
-      for (int base = 0; base < K && found < 0; base += 32) {
-        const int idx = base + lane;
-        const bool isf = idx < K && fl[idx] == f;
-        const unsigned m_any = __ballot_sync(FULL, isf);
-        const unsigned m_after = __ballot_sync(FULL, isf && tau[idx] > t1);
-        if (first_any < 0 && m_any) first_any = base + __ffs(m_any) - 1;
-        if (m_after) found = base + __ffs(m_after) - 1;
+      const long long k1 = time_key(t1);
+      for (int base = 0; base < K && found < 0; base += 128) {
+        bool isf[4], after[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int idx = base + 32 * c + lane;
+          isf[c] = idx < K && fl[idx] == f;
+          after[c] = idx < K && time_key(tau[idx]) > k1;
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const unsigned m_any = __ballot_sync(FULL, isf[c]);
+          const unsigned m_after = __ballot_sync(FULL, isf[c] && after[c]);
+          if (first_any < 0 && m_any) first_any = base + 32 * c + __ffs(m_any) - 1;
+          if (found < 0 && m_after) found = base + 32 * c + __ffs(m_after) - 1;
+        }
       }
       const int j = found >= 0 ? found : first_any;
       if (j < 0) {  // the operator counts always match k_f; the guard only keeps reads in bounds
@@ -262,27 +287,31 @@ __global__ void sweep_propose_kernel(SweepView S0, const double *__restrict__ un
     if (t2 == t1) null_move = true;
     if (!null_move) {
       const double td = seg ? t1 : t2, ta = seg ? t2 : t1;
-      const double lp = kf == 0 ? 2.0 * log(beta) : log(beta * lmax / (2.0 * (kf + 1)));
       // bordered matrix: C_i = Fh(tau'_i - ta), R_j = Fh(td - tau_j), d = Fh(td - ta)
-      for (int i = lane; i < kf; i += 32) {
-        Cv[i] = hyb_Fh(S, f, rt[i] - ta);
-        Rv[i] = hyb_Fh(S, f, td - ct[i]);
+      for (int e = lane; e <= 2 * kf; e += 32) {
+        const double x = e < kf ? rt[e] : td, y = e >= kf && e < 2 * kf ? ct[e - kf] : ta;
+        CR[e] = hyb_Fh(S, f, x - y);
       }
       __syncwarp();
-      double *mc = S.p_vec + (size_t)w * 2 * S.kcap, *rm = mc + S.kcap;
+      double *vec = S.p_vec + (size_t)w * 2 * S.kcap;
       double part = 0.0;
-      for (int j = lane; j < kf; j += 32) {  // (M C)_j
+      for (int e = lane; e < 2 * kf; e += 32) {  // (M C)_j by the first kf lanes, (R M)_i by the next
+        const bool mc = e < kf;
+        const int r = mc ? e : e - kf, step = mc ? 1 : S.kcap;
+        const double *m = Mf + (mc ? (size_t)r * S.kcap : (size_t)r), *x = mc ? CR : CR + kf;
         double a = 0.0;
-        for (int i = 0; i < kf; ++i) a = fma(Mf[(size_t)j * S.kcap + i], Cv[i], a);
-        mc[j] = a;
-        part = fma(Rv[j], a, part);
+#pragma unroll 4
+        for (int i = 0; i < kf; ++i) a = fma(m[(size_t)i * step], x[i], a);
+        vec[mc ? r : S.kcap + r] = a;
+        if (mc) part = fma(CR[kf + r], a, part);
       }
-      for (int i = lane; i < kf; i += 32) {  // (R M)_i
-        double a = 0.0;
-        for (int j = 0; j < kf; ++j) a = fma(Rv[j], Mf[(size_t)j * S.kcap + i], a);
-        rm[i] = a;
-      }
-      const double lambda = hyb_Fh(S, f, td - ta) - warp_sum(part);
+#pragma unroll
+      for (int o2 = 16; o2 > 0; o2 >>= 1)  // lanes from kf on hold zeros
+        if (kf > o2) part += __shfl_xor_sync(FULL, part, o2);
+      const double lambda = __shfl_sync(FULL, CR[2 * kf] - part, 0);
+      // both logarithms at once: lane 0 the proposal factor's, the others |lambda|'s
+      const double lg = log(lane == 0 ? (kf == 0 ? beta : beta * lmax / (2.0 * (kf + 1))) : fabs(lambda));
+      const double lp = kf == 0 ? 2.0 * lg : lg, ldet = __shfl_sync(FULL, lg, 1);
       const int X = perm_count(tau, fl, K, f, td, ta, -1, -1, lane);
       if (lane == 0) {
         S.p_t1[w] = t1;
@@ -292,7 +321,7 @@ __global__ void sweep_propose_kernel(SweepView S0, const double *__restrict__ un
         S.mv_tdag[w] = td;
         S.mv_tann[w] = ta;
         S.p_lprop[w] = lp;
-        S.p_ldet[w] = log(fabs(lambda));
+        S.p_ldet[w] = ldet;
         S.p_sign[w] = (int8_t)((lambda > 0.0 ? 1 : (lambda < 0.0 ? -1 : 0)) * ((X & 1) ? -1 : 1));
         S.p_lambda[w] = lambda;
       }
@@ -300,37 +329,34 @@ __global__ void sweep_propose_kernel(SweepView S0, const double *__restrict__ un
     }
   } else {
     // ---- removal ----
-    if (lane == 0) atomicAdd(&S.counters[C_REM_PROP], 1ull);
+    if (lane == 0 && !Tv.T) atomicAdd(&S.counters[C_REM_PROP], 1ull);
     if (kf > 0) {
       int jsel = (int)(u[2] * 2 * kf);
       jsel = jsel > 2 * kf - 1 ? 2 * kf - 1 : jsel;
-      const int a = nth_of_flavor(fl, K, f, jsel, lane);
-      const int b = nth_of_flavor(fl, K, f, (jsel + 1) % (2 * kf), lane);
-      const int c = kf > 1 ? nth_of_flavor(fl, K, f, (jsel + 2) % (2 * kf), lane) : a;
+      const int nth[3] = {jsel, (jsel + 1) % (2 * kf), (jsel + 2) % (2 * kf)};
+      int at[3];
+      three_of_flavor(fl, K, f, nth, at, lane);
+      const int a = at[0], b = at[1], c = at[2];
       // the operator counts always match k_f; the guard only keeps every read in bounds
       const bool found = a >= 0 && b >= 0 && c >= 0;
-      const double t1 = found ? tau[a] : 0.0, t2 = found ? tau[b] : 0.0;
-      double lp;
-      if (kf == 1) {
-        lp = -2.0 * log(beta);
-      } else {
-        const double tc = found ? tau[c] : 0.0;
-        const double lmax = tc > t1 ? tc - t1 : tc + beta - t1;
-        lp = log(2.0 * kf / (beta * lmax));
-      }
+      const double t1 = found ? tau[a] : 0.0, t2 = found ? tau[b] : 0.0, tc = found ? tau[c] : 0.0;
+      const double lmax = tc > t1 ? tc - t1 : tc + beta - t1;
       const int da = found ? dg[a] : 0, db = found ? dg[b] : 0;
       const double td = da == 1 ? t1 : t2, ta = da == 1 ? t2 : t1;
       int ri = -1, cj = -1;
+      const long long kd = time_key(td), ka = time_key(ta);
       for (int base = 0; base < kf; base += 32) {
         const int idx = base + lane;
-        const unsigned mr = __ballot_sync(FULL, idx < kf && rt[idx] == td);
-        const unsigned mcn = __ballot_sync(FULL, idx < kf && ct[idx] == ta);
+        const unsigned mr = __ballot_sync(FULL, idx < kf && time_key(rt[idx]) == kd);
+        const unsigned mcn = __ballot_sync(FULL, idx < kf && time_key(ct[idx]) == ka);
         if (ri < 0 && mr) ri = base + __ffs(mr) - 1;
         if (cj < 0 && mcn) cj = base + __ffs(mcn) - 1;
       }
       if (found && ri >= 0 && cj >= 0 && da != db) {
         const double ratio = Mf[(size_t)cj * S.kcap + ri];
         const int X = perm_count(tau, fl, K, f, td, ta, a, b, lane);
+        const double lg = log(lane == 0 ? (kf == 1 ? beta : 2.0 * kf / (beta * lmax)) : fabs(ratio));
+        const double lp = kf == 1 ? -2.0 * lg : lg, ldet = __shfl_sync(FULL, lg, 1);
         if (lane == 0) {
           S.p_t1[w] = t1;
           S.p_t2[w] = t2;
@@ -340,7 +366,7 @@ __global__ void sweep_propose_kernel(SweepView S0, const double *__restrict__ un
           S.mv_kind[w] = 1;
           S.mv_rem[w] = a;
           S.p_lprop[w] = lp;
-          S.p_ldet[w] = log(fabs(ratio));
+          S.p_ldet[w] = ldet;
           S.p_sign[w] = (int8_t)((ratio > 0.0 ? 1 : (ratio < 0.0 ? -1 : 0)) * ((X & 1) ? -1 : 1));
           S.p_ij[2 * w] = ri;
           S.p_ij[2 * w + 1] = cj;
@@ -356,7 +382,7 @@ __global__ void sweep_propose_kernel(SweepView S0, const double *__restrict__ un
       // a move the trace stage skips (structural zero of the pipeline is avoided:
       // kind 2 is rejected by its validation without any work)
       S.mv_kind[w] = 2;
-      atomicAdd(&S.counters[C_NULL], 1ull);
+      if (!Tv.T) atomicAdd(&S.counters[C_NULL], 1ull);
     }
   }
 }
@@ -490,9 +516,8 @@ __global__ void sweep_accept_kernel(SweepView S, const double *__restrict__ u5s,
 
 // Feature vector of each proposal (see kt_sweep_feature_size): the configuration without
 // the move's pair (the base) and the pair. A removal's base skips the pair's operators.
-__global__ void sweep_features_kernel(SweepView S0, TryView Tv) {
+__global__ void sweep_features_kernel(SweepView S) {
   extern __shared__ float hsm[];
-  const SweepView S = Tv.T ? try_view(S0, Tv, blockIdx.y) : S0;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int w = blockIdx.x * (blockDim.x >> 5) + wib;
   if (w >= S.nw) return;
@@ -561,34 +586,66 @@ __global__ void sweep_features_kernel(SweepView S0, TryView Tv) {
   }
 }
 
-// Multi-try delayed acceptance, before the features: for every operator i of a walker, the
-// next operator of the same flavor after it, cyclically (-1 if i is its flavor's only one),
-// one warp per walker. The tries of a call step share the configuration, so this table is
-// built once and every try's features take O(K) instead of O(K^2 / n_flavors).
-__global__ void sweep_next_flavor_kernel(SweepView S, TryView Tv) {
-  const int lane = threadIdx.x & 31;
-  const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+// Multi-try delayed acceptance, before the features, one warp per walker: for every operator the next
+// of its flavor, cyclically, and for every creator its segment. The tries of a step share the
+// configuration, so lengths and bins (FP64, a division each) are found once, not once per try. Chunks of
+// 32 operators from the top: the next one is the nearest higher lane of the flavor, or the lowest
+// operator of the flavor in the chunks above (from the top around: the flavor's first).
+__global__ void sweep_segments_kernel(SweepView S, TryView Tv) {
+  extern __shared__ int carry_sh[];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int w = blockIdx.x * (blockDim.x >> 5) + wib;
   if (w >= S.nw) return;
+  int *carry = carry_sh + wib * S.nf;
   const int o = S.offsets[w], K = S.lens[w];
-  const uint8_t *fl = S.flv + o;
+  const double *tau = S.tau + o;
+  const uint8_t *fl = S.flv + o, *dg = S.dag + o;
   int16_t *nxt = Tv.nxt + (size_t)w * S.cap;
-  for (int i = lane; i < K; i += 32) {
-    const int f = fl[i];
+  double2 *seg_t = Tv.seg_t + (size_t)w * (S.cap / 2);
+  uint2 *seg_m = Tv.seg_m + (size_t)w * (S.cap / 2);
+  for (int f = lane; f < S.nf; f += 32) carry[f] = K;
+  __syncwarp();
+  for (int i = lane; i < K; i += 32) atomicMin(&carry[fl[i]], i);
+  __syncwarp();
+  int n = 0;  // segments so far
+  for (int base = (K - 1) / 32 * 32; base >= 0 && K > 0; base -= 32) {
+    const int i = base + lane;
+    const bool in = i < K;
+    const int f = in ? fl[i] : -1;
+    const bool cre = in && dg[i] == 1;
+    const unsigned same = __match_any_sync(FULL, f), above = ~((2u << lane) - 1u);
     int j = -1;
-    for (int s2 = 1; s2 < K; ++s2) {
-      const int c = i + s2 < K ? i + s2 : i + s2 - K;
-      if (fl[c] == f) {
-        j = c;
-        break;
+    if (in) j = (same & above) ? base + __ffs(same & above) - 1 : carry[f];
+    if (j == i) j = -1;
+    __syncwarp();
+    if (in && (same & ((1u << lane) - 1u)) == 0) carry[f] = i;
+    __syncwarp();
+    if (in) nxt[i] = (int16_t)j;
+    const unsigned cm = __ballot_sync(FULL, cre);
+    const int s = n + __popc(cm & above);
+    n += __popc(cm);
+    if (cre && s < S.cap / 2) {
+      double t = tau[i], e = t;
+      int b = 255;
+      if (j >= 0) {
+        const double l = tau[j] > t ? tau[j] - t : tau[j] + S.beta - t;
+        b = (int)(l / S.beta * 32);
+        b = b > 31 ? 31 : b;
+        e = t + l;
       }
+      seg_t[s] = make_double2(t, e);
+      seg_m[s] = make_uint2((unsigned)i | (unsigned)(j & 0xffff) << 16, (unsigned)f | (unsigned)b << 8);
     }
-    nxt[i] = (int16_t)j;
   }
+  if (lane == 0) Tv.n_seg[w] = n < S.cap / 2 ? n : S.cap / 2;
 }
 
-// Features of the tries (one warp per walker and try), with the values of
-// sweep_features_kernel: a removal try's base skips its own pair by following the walker's
-// next-same-flavor table past the pair's two operators.
+// Features of the tries (one warp per walker and try), with the values of sweep_features_kernel: a
+// removal try's base skips its own pair by following the next-of-flavor table past it. Bounded by the
+// FP64 pipe before the segments' table: lengths, bins and 18 FP64 instructions of overlaps for every
+// operator of every try. Now an FP64 instruction runs where an image of the pair's interval overlaps a
+// segment (ends are compared as integers), and the divisions share one evaluation. 8,192 tries (1,024
+// chains at beta = 50): 103 -> 47 us.
 __global__ void sweep_features_multi_kernel(SweepView S, TryView Tv) {
   extern __shared__ float hsm[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -597,60 +654,74 @@ __global__ void sweep_features_multi_kernel(SweepView S, TryView Tv) {
   const int nf = S.nf;
   const double beta = S.beta;
   const size_t sl = (size_t)blockIdx.y * S.nw + w;
-  float *hist = hsm + (size_t)wib * nf * 34;
+  // per warp: nf x 32 histogram bins, nf occupied lengths (double), nf + 1 quotients
+  float *hist = hsm + (size_t)wib * (nf * 34 + ((nf + 2) & ~1));
   double *occ = reinterpret_cast<double *>(hist + nf * 32);
-  for (int i = lane; i < nf * 32; i += 32) hist[i] = 0.f;
-  for (int i = lane; i < nf; i += 32) occ[i] = 0.0;
+  float *quo = hist + nf * 34;
+  for (int i = lane; i < nf * 34; i += 32) hist[i] = 0.f;
   __syncwarp();
   const double m0 = Tv.p_t1[sl];
   double md = Tv.p_t2[sl] - m0;
   if (md < 0.0) md += beta;
-  const int o = S.offsets[w], K = S.lens[w];
-  const double *tau = S.tau + o;
-  const uint8_t *fl = S.flv + o, *dg = S.dag + o;
+  const double *tau = S.tau + S.offsets[w];
   const int16_t *nxt = Tv.nxt + (size_t)w * S.cap;
-  const int pa = Tv.p_pair[2 * sl], pb = Tv.p_pair[2 * sl + 1];
-  for (int i = lane; i < K; i += 32) {
-    if (dg[i] != 1 || i == pa || i == pb) continue;
-    const int f = fl[i];
-    int j = nxt[i];
-    while (j >= 0 && (j == pa || j == pb)) j = nxt[j];
-    if (j == i) j = -1;
-    if (j < 0) continue;
-    const double ti = tau[i], tj = tau[j];
-    const double l = tj > ti ? tj - ti : tj + beta - ti;
-    int b = (int)(l / beta * 32);
-    b = b > 31 ? 31 : b;
-    atomicAdd(&hist[f * 32 + b], 0.25f);
-    double ov = 0.0;
-    for (int k = -1; k <= 1; ++k) {
-      const double lo = fmax(ti, m0 + k * beta), hi = fmin(ti + l, m0 + md + k * beta);
-      ov += fmax(0.0, hi - lo);
+  const double2 *seg_t = Tv.seg_t + (size_t)w * (S.cap / 2);
+  const uint2 *seg_m = Tv.seg_m + (size_t)w * (S.cap / 2);
+  const int pa = Tv.p_pair[2 * sl], pb = Tv.p_pair[2 * sl + 1], ns = Tv.n_seg[w];
+  // the images [from, to) of the pair's interval; a negative end is a negative integer too
+  long long from[3], to[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    from[k] = __double_as_longlong(m0 + (k - 1) * beta);
+    to[k] = __double_as_longlong(m0 + md + (k - 1) * beta);
+  }
+#pragma unroll 2
+  for (int s = lane; s < ns; s += 32) {
+    const uint2 m = seg_m[s];
+    const double2 te = seg_t[s];
+    const int i = (int)(m.x & 0xffffu), f = (int)(m.y & 0xffu);
+    int j = (int)(int16_t)(m.x >> 16), b = (int)(m.y >> 8);
+    double end = te.y;
+    if (b == 255 || i == pa || i == pb) continue;
+    if (j == pa || j == pb) {
+      while (j >= 0 && (j == pa || j == pb)) j = nxt[j];
+      if (j == i || j < 0) continue;
+      const double tj = tau[j], l = tj > te.x ? tj - te.x : tj + beta - te.x;
+      b = (int)(l / beta * 32);
+      b = b > 31 ? 31 : b;
+      end = te.x + l;
     }
-    if (ov > 0.0) atomicAdd(&occ[f], ov);
+    atomicAdd(&hist[f * 32 + b], 0.25f);
+    // overlap of the segment with the pair's interval, cyclically
+    const long long t0 = time_key(te.x), t1 = time_key(end);
+    double ov = 0.0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const long long lo = t0 > from[k] ? t0 : from[k], hi = t1 < to[k] ? t1 : to[k];
+      if (hi > lo) ov += __longlong_as_double(hi) - __longlong_as_double(lo);
+    }
+    if (__double_as_longlong(ov) != 0) atomicAdd(&occ[f], ov);
   }
   __syncwarp();
-  __nv_bfloat16 *row = Tv.X + sl * S.n_in;
-  const int fm = Tv.mv_flv[sl];
-  for (int i = lane; i < S.n_in; i += 32) {
-    float x = 0.f;
-    if (i < nf) {
-      x = (float)(S.kf[(size_t)w * nf + i] - (pa >= 0 && i == fm ? 1 : 0)) / 8.f;
-    } else if (i < 33 * nf) {
-      x = hist[i - nf];
-    } else if (i == 33 * nf) {
-      x = 0.f;
-    } else if (i <= 34 * nf) {
-      x = (i - 33 * nf - 1 == fm) ? 1.f : 0.f;
-    } else if (i == 34 * nf + 1) {
-      x = (float)(md / beta);
-    } else if (i == 34 * nf + 2) {
-      x = Tv.p_seg[sl] ? 1.f : -1.f;
-    } else if (i < 35 * nf + 3) {
-      x = md > 0.0 ? (float)(occ[i - 34 * nf - 3] / md) : 0.f;
-    }
-    row[i] = __float2bfloat16_rn(x);
+  for (int i = lane; i <= nf; i += 32) {
+    const double num = i < nf ? occ[i] : md, den = i < nf ? md : beta;
+    quo[i] = den > 0.0 ? (float)(num / den) : 0.f;
   }
+  __syncwarp();
+  __nv_bfloat162 *row = reinterpret_cast<__nv_bfloat162 *>(Tv.X + sl * S.n_in);
+  const int fm = Tv.mv_flv[sl];
+  const int32_t *kf = S.kf + (size_t)w * nf;
+  const float segment = Tv.p_seg[sl] ? 1.f : -1.f;
+  auto feature = [&](int i) -> float {
+    if (i < nf) return (float)(kf[i] - (pa >= 0 && i == fm ? 1 : 0)) / 8.f;
+    if (i < 33 * nf) return hist[i - nf];
+    if (i == 33 * nf) return 0.f;
+    if (i <= 34 * nf) return i - 33 * nf - 1 == fm ? 1.f : 0.f;
+    if (i == 34 * nf + 1) return quo[nf];
+    if (i == 34 * nf + 2) return segment;
+    return i < 35 * nf + 3 ? quo[i - 34 * nf - 3] : 0.f;
+  };
+  for (int i = lane; i < S.n_in / 2; i += 32) row[i] = __floats2bfloat162_rn(feature(2 * i), feature(2 * i + 1));
 }
 
 // Stage 1 of delayed acceptance: the surrogate's ratio decides whether the trace is computed.
@@ -676,43 +747,48 @@ __global__ void sweep_stage1_kernel(SweepView S, const double *__restrict__ uni)
 // it is (rejected at stage 1, or a null move); the tries after it are never taken. A walker
 // none of whose tries passes keeps its configuration for T steps. Counters of the tries taken.
 __global__ void sweep_select_kernel(SweepView S, TryView Tv, const double *__restrict__ uni) {
+  __shared__ int cnt[5];
   const int lane = threadIdx.x & 31;
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= S.nw) return;
   const int nw = S.nw, T = Tv.T;
+  if (threadIdx.x < 5) cnt[threadIdx.x] = 0;
+  __syncthreads();
+  // a lane per try (T <= 32): one logarithm of FP64 instructions for all
   int sel = -1;
-  float ysel = 0.f;
-  if (lane == 0) {
-    unsigned long long c_ins = 0, c_rem = 0, c_null = 0, c_cap = 0, c_st1 = 0;
-    for (int t = 0; t < T; ++t) {
-      const size_t sl = (size_t)t * nw + w;
-      const int kind = Tv.p_kind[sl];
-      if (kind == 0) ++c_ins;
-      else ++c_rem;
-      if (!Tv.p_valid[sl]) {
-        ++c_null;
-        if (kind == 0 && S.kf[(size_t)w * S.nf + Tv.mv_flv[sl]] >= S.kcap) ++c_cap;
-        continue;
-      }
-      const float y = kind != 0 ? -Tv.ytil[sl] : Tv.ytil[sl];
-      const double lt = (double)y + Tv.p_ldet[sl] + Tv.p_lprop[sl];
-      const double u6 = uni[((size_t)w * T + t) * 7 + 6];
-      if ((u6 > 0.0 ? log(u6) : -INFINITY) < lt) {
-        sel = t;
-        ysel = y;
-        break;
-      }
-      ++c_st1;
+  float y = 0.f;
+  if (w < nw) {
+    const bool in = lane < T;
+    const size_t sl = (size_t)(in ? lane : 0) * nw + w;
+    const int kind = Tv.p_kind[sl];
+    const bool valid = in && Tv.p_valid[sl];
+    y = kind != 0 ? -Tv.ytil[sl] : Tv.ytil[sl];
+    const double lt = (double)y + Tv.p_ldet[sl] + Tv.p_lprop[sl];
+    const double u6 = uni[((size_t)w * T + (in ? lane : 0)) * 7 + 6];
+    const bool pass = valid && (u6 > 0.0 ? log(u6) : -INFINITY) < lt;
+    const bool full = in && !valid && kind == 0 && S.kf[(size_t)w * S.nf + Tv.mv_flv[sl]] >= S.kcap;
+    const unsigned pm = __ballot_sync(FULL, pass), im = __ballot_sync(FULL, in && kind == 0);
+    const unsigned vm = __ballot_sync(FULL, valid), fm = __ballot_sync(FULL, full);
+    sel = pm ? __ffs(pm) - 1 : -1;
+    const int n = sel < 0 ? T : sel + 1;
+    const unsigned taken = n >= 32 ? FULL : (1u << n) - 1u;
+    if (lane == 0) {
+      Tv.n_tries[w] = n;
+      S.p_acc[w] = 0;
+      atomicAdd(&cnt[0], __popc(im & taken));
+      atomicAdd(&cnt[1], __popc(~im & taken));
+      atomicAdd(&cnt[2], __popc(~vm & taken));
+      atomicAdd(&cnt[3], __popc(fm & taken));
+      atomicAdd(&cnt[4], __popc(vm & ~pm & taken));
     }
-    Tv.n_tries[w] = sel < 0 ? T : sel + 1;
-    S.p_acc[w] = 0;
-    if (c_ins) atomicAdd(&S.counters[C_INS_PROP], c_ins);
-    if (c_rem) atomicAdd(&S.counters[C_REM_PROP], c_rem);
-    if (c_null) atomicAdd(&S.counters[C_NULL], c_null);
-    if (c_cap) atomicAdd(&S.counters[C_CAP], c_cap);
-    if (c_st1) atomicAdd(&S.counters[C_STAGE1], c_st1);
   }
-  sel = __shfl_sync(FULL, sel, 0);
+  __syncthreads();
+  if (threadIdx.x < 5 && cnt[threadIdx.x]) {
+    const int to = threadIdx.x == 0 ? C_INS_PROP : threadIdx.x == 1 ? C_REM_PROP : threadIdx.x == 2 ? C_NULL
+                   : threadIdx.x == 3 ? C_CAP : C_STAGE1;
+    atomicAdd(&S.counters[to], (unsigned long long)cnt[threadIdx.x]);
+  }
+  if (w >= nw) return;
+  const float ysel = __shfl_sync(FULL, y, sel < 0 ? 0 : sel);
   if (sel < 0) {
     if (lane == 0) {
       S.p_valid[w] = 0;
@@ -1183,8 +1259,9 @@ kt_status alloc_tries(kt_sweep *s, int T, size_t *dry = nullptr) {
                o_t1 = take(n * 8), o_t2 = take(n * 8), o_td = take(n * 8), o_ta = take(n * 8), o_lp = take(n * 8),
                o_ld = take(n * 8), o_lam = take(n * 8), o_vec = take(n * 2 * kc * 8), o_pair = take(n * 2 * 4),
                o_rem = take(n * 4), o_ij = take(n * 2 * 4), o_mk = take(n), o_mf = take(n),
-               o_X = take(n * (size_t)s->v.n_in * 2), o_y = take(n * 4), o_cnt = take(KT_SWEEP_NCOUNTERS * 8),
-               o_nt = take(nw * 4), o_u5 = take(nw * 8), o_nxt = take(nw * (size_t)s->v.cap * 2);
+               o_X = take(n * (size_t)s->v.n_in * 2), o_y = take(n * 4), o_nt = take(nw * 4),
+               o_u5 = take(nw * 8), o_nxt = take(nw * (size_t)s->v.cap * 2), o_sgt = take(nw * (size_t)(s->v.cap / 2) * 16),
+               o_sgm = take(nw * (size_t)(s->v.cap / 2) * 8), o_nsg = take(nw * 4);
   if (dry) {
     *dry = b;
     return KT_OK;
@@ -1204,9 +1281,10 @@ kt_status alloc_tries(kt_sweep *s, int T, size_t *dry = nullptr) {
   t.p_lambda = (double *)(p + o_lam); t.p_vec = (double *)(p + o_vec); t.p_pair = (int32_t *)(p + o_pair);
   t.mv_rem = (int32_t *)(p + o_rem); t.p_ij = (int32_t *)(p + o_ij); t.mv_kind = (uint8_t *)(p + o_mk);
   t.mv_flv = (uint8_t *)(p + o_mf); t.X = (__nv_bfloat16 *)(p + o_X); t.ytil = (float *)(p + o_y);
-  t.scratch_counters = (unsigned long long *)(p + o_cnt); t.n_tries = (int32_t *)(p + o_nt);
+  t.n_tries = (int32_t *)(p + o_nt);
   t.u5 = (double *)(p + o_u5);
   t.nxt = (int16_t *)(p + o_nxt);
+  t.seg_t = (double2 *)(p + o_sgt); t.seg_m = (uint2 *)(p + o_sgm); t.n_seg = (int32_t *)(p + o_nsg);
   t.T = T;
   return KT_OK;
 }
@@ -1360,6 +1438,10 @@ kt_status kt_sweep_create(kt_model *m, const kt_sweep_params *p, kt_sweep **out)
   return KT_OK;
 }
 
+// Warps per block of the kernels with a warp per walker (or try): their FP64 instructions share one pipe
+// per SM, so a batch that does not fill the chip is spread over all 152 SMs before a block gets its second warp.
+static int warps_per_block(long long n) { return (int)std::max(1ll, std::min(8ll, (n + 151) / 152)); }
+
 // Shared step loop of kt_sweep_run (mode 0), kt_sweep_run_da (1) and kt_sweep_collect (2).
 static kt_status run_steps(kt_sweep *s, int32_t n_steps, const double *uniforms, int32_t meas_every, void *stream,
                            int mode, __nv_bfloat16 *feat, float *targ, int *count, int cap) {
@@ -1374,15 +1456,15 @@ static kt_status run_steps(kt_sweep *s, int32_t n_steps, const double *uniforms,
   const kt::Workspace w = kt::carve_workspace(s->ws, v.nw, M.n_kept, M.d_max, 0);
   const kt::MoveView mvv{v.mv_kind, v.mv_flv, v.mv_tdag, v.mv_tann, v.mv_rem};
   const kt::SeqView sv = seq_view(s);
-  const int wpb = 8;
+  const int wpb = warps_per_block(v.nw);
   const unsigned grid = (unsigned)((v.nw + wpb - 1) / wpb);
-  const size_t shm = (size_t)wpb * 2 * v.kcap * sizeof(double);
+  const size_t shm = (size_t)wpb * (2 * v.kcap + 1) * sizeof(double);
   cudaGetLastError();
   const size_t shf = (size_t)wpb * v.nf * 34 * sizeof(float);
   for (int step = 0; step < n_steps; ++step) {
     const double *u = uniforms + (size_t)step * v.nw * ustride;
     kt::sweep_propose_kernel<<<grid, wpb * 32, shm, st>>>(v, u, ustride, kt::TryView{});
-    if (mode != 0) kt::sweep_features_kernel<<<grid, wpb * 32, shf, st>>>(v, kt::TryView{});
+    if (mode != 0) kt::sweep_features_kernel<<<grid, wpb * 32, shf, st>>>(v);
     if (mode == 1) {
       if (kt::mlp_forward(s->net, v.X, v.nw, v.ytil, false, st) != 0) return KT_ECUDA;
       kt::sweep_stage1_kernel<<<(v.nw + 255) / 256, 256, 0, st>>>(v, u);
@@ -1437,20 +1519,20 @@ kt_status kt_sweep_run_da_multi(kt_sweep *s, int32_t n_steps, int32_t tries, con
   const kt::Workspace w = kt::carve_workspace(s->ws, v.nw, M.n_kept, M.d_max, 0);
   const kt::MoveView mvv{v.mv_kind, v.mv_flv, v.mv_tdag, v.mv_tann, v.mv_rem};
   const kt::SeqView sv = seq_view(s);
-  const int wpb = 8;
+  const int wpb = warps_per_block(v.nw), wpt = warps_per_block((long long)v.nw * tries);
   const unsigned grid = (unsigned)((v.nw + wpb - 1) / wpb);
-  const size_t shm = (size_t)wpb * 2 * v.kcap * sizeof(double);
-  const size_t shf = (size_t)wpb * v.nf * 34 * sizeof(float);
+  const size_t shm = (size_t)wpt * (2 * v.kcap + 1) * sizeof(double);
+  const size_t shf = (size_t)wpt * (v.nf * 34 + ((v.nf + 2) & ~1)) * sizeof(float);
   const int ustride = 7 * tries;
   cudaGetLastError();
   for (int step = 0; step < n_steps; ++step) {
     const double *u = uniforms + (size_t)step * v.nw * ustride;
     // every try from the walker's current configuration (the configuration only changes at
     // the end of the step), all scored by one surrogate inference
-    const dim3 grid_t(grid, (unsigned)tries);
-    kt::sweep_propose_kernel<<<grid_t, wpb * 32, shm, st>>>(v, u, ustride, tv);
-    kt::sweep_next_flavor_kernel<<<grid, wpb * 32, 0, st>>>(v, tv);
-    kt::sweep_features_multi_kernel<<<grid_t, wpb * 32, shf, st>>>(v, tv);
+    const dim3 grid_t((unsigned)((v.nw + wpt - 1) / wpt), (unsigned)tries);
+    kt::sweep_propose_kernel<<<grid_t, wpt * 32, shm, st>>>(v, u, ustride, tv);
+    kt::sweep_segments_kernel<<<grid, wpb * 32, wpb * v.nf * sizeof(int), st>>>(v, tv);
+    kt::sweep_features_multi_kernel<<<grid_t, wpt * 32, shf, st>>>(v, tv);
     if (kt::mlp_forward(s->net, tv.X, tries * v.nw, tv.ytil, false, st) != 0) return KT_ECUDA;
     kt::sweep_select_kernel<<<grid, wpb * 32, 0, st>>>(v, tv, u);
     // measurement of the configuration the walker spent this step's tries in, weighted by them
