@@ -94,9 +94,9 @@ __device__ __forceinline__ float2 eig_weight_pair(float2 lam, const EigDt &dt, c
   float xl = fmaf(dt.h, lam.x, -xh);
   xl = fmaf(dt.h, lam.y, xl);
   xl = fmaf(dt.l, lam.x, xl);
-  const float t = rintf(-32.f * xh);
-  const int i = (int)t;
-  const float f = fmaf(t, -0.03125f, -xh);  // exact
+  const float t = fmaf(xh, -32.f, 12582912.f);  // 1.5 * 2^23: rounded to an integer in the low bits
+  const int i = __float_as_int(t) - 0x4b400000;
+  const float f = fmaf(t - 12582912.f, -0.03125f, -xh);  // exact
   const float L2H = 0.693147182f, L2L = -1.90465421e-9f;  // ln 2 as a pair
   const float rh = f * L2H;
   float rl = fmaf(f, L2H, -rh);
@@ -213,7 +213,17 @@ __device__ __forceinline__ float2 eig_mul_pair(float2 x, float2 w) {
   return make_float2(h, pe - (h - p));
 }
 
-// x (EIG_PAIR: any pair) times the weights of an interval dt in the block whose first
+template <int MODE>
+__device__ __forceinline__ typename EigT<MODE>::E eig_lambda(const DevModel &M, int at) {
+  return __ldg((const typename EigT<MODE>::E *)M.eig_lam + at);
+}
+template <int MODE>
+__device__ __forceinline__ typename EigT<MODE>::E eig_weight(const DevModel &M, typename EigT<MODE>::E lam, const EigDt &dt) {
+  if constexpr (MODE == EIG_PAIR) return eig_weight_pair(lam, dt, (const float2 *)M.eig_tab);
+  else return eig_weight_f64(lam, dt.d, (const double *)M.eig_tab);
+}
+
+// x (EIG_PAIR: any pair) times the weights wt of an interval dt in the block whose first
 // eigenvalue is at eoff. The weights are relative to the block's lowest eigenvalue. When that
 // leaves every component small (a vector without components on the low eigenvalues, or a
 // small matrix element), the weights are formed again relative to the lowest eigenvalue that
@@ -222,8 +232,9 @@ __device__ __forceinline__ float2 eig_mul_pair(float2 x, float2 w) {
 // which costs no reduction and no wait. False if the vector is exactly zero. `act`: the group
 // has such an interval (the others keep x); all lanes of the warp call it together.
 template <int MODE, int G, int R>
-__device__ __forceinline__ bool eig_interval(const DevModel &M, typename EigT<MODE>::E (&x)[R], bool act, int gl,
-                                             int eoff, int d, const EigDt &dt, double &Lx, int &ex, float &sc) {
+__device__ __forceinline__ bool eig_interval(const DevModel &M, typename EigT<MODE>::E (&x)[R],
+                                             const typename EigT<MODE>::E (&wt)[R], bool act, int gl, int eoff, int d,
+                                             const EigDt &dt, double &Lx, int &ex, float &sc) {
   using E = typename EigT<MODE>::E;
   E y[R];
   bool large = false, big = false;
@@ -233,13 +244,10 @@ __device__ __forceinline__ bool eig_interval(const DevModel &M, typename EigT<MO
     y[j] = eig_zero<MODE>();
     if (r < d) {
       if constexpr (MODE == EIG_PAIR) {
-        float2 w = eig_weight_pair(__ldg((const float2 *)M.eig_lam + eoff + r), dt, (const float2 *)M.eig_tab);
-        w.x *= sc;
-        w.y *= sc;
-        y[j] = eig_mul_pair(x[j], w);
+        y[j] = eig_mul_pair(x[j], make_float2(wt[j].x * sc, wt[j].y * sc));
         big |= fabsf(y[j].x) >= 0.0625f;
       } else {
-        y[j] = x[j] * eig_weight_f64(__ldg((const double *)M.eig_lam + eoff + r), dt.d, (const double *)M.eig_tab);
+        y[j] = x[j] * wt[j];
       }
     }
     large |= eig_large<MODE>(y[j]);
@@ -308,6 +316,19 @@ __device__ __forceinline__ bool eig_interval(const DevModel &M, typename EigT<MO
     }
   }
   return alive;
+}
+
+// EIG_PAIR, blocks of at most 12 rows: the same with the three small products in sums of their own, which
+// leaves chains of two FMAs a vector where one sum makes a chain of six.
+__device__ __forceinline__ void eig_fma4(float (&a)[4], const float4 &m, const float4 &v) {
+  a[0] = fmaf(m.x, v.x, a[0]);
+  a[1] = fmaf(m.x, v.y, a[1]);
+  a[2] = fmaf(m.y, v.x, a[2]);
+  a[3] = fmaf(m.y, v.y, a[3]);
+  a[0] = fmaf(m.z, v.z, a[0]);
+  a[1] = fmaf(m.z, v.w, a[1]);
+  a[2] = fmaf(m.w, v.z, a[2]);
+  a[3] = fmaf(m.w, v.w, a[3]);
 }
 
 // One 16-byte vector of a row of an operator matrix (two entries) times the vector in shared
@@ -464,7 +485,11 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
     if (act) L0 = fma(-dt.d, __ldg(M.eig_base + u.b), L0);
     dt.h = (float)dt.d;
     dt.l = (float)(dt.d - (double)dt.h);
-    if (!eig_interval<MODE, G, R>(M, u.x, act, gl, __ldg(M.blk_off + u.b), u.dim, dt, Lx, ex, sc)) u.vanished = true;
+    const int eo = __ldg(M.blk_off + u.b);
+    E wt[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) wt[j] = gl + G * j < u.dim ? eig_weight<MODE>(M, eig_lambda<MODE>(M, eo + gl + G * j), dt) : eig_zero<MODE>();
+    if (!eig_interval<MODE, G, R>(M, u.x, wt, act, gl, eo, u.dim, dt, Lx, ex, sc)) u.vanished = true;
   }
   const int key = __ldg(M.blk_key + u.b);
   int nn = key & 0xfffff, mk = key >> 20;
@@ -477,19 +502,52 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
   const int nmax = G == 32 ? n : __reduce_max_sync(FULL, n);
   int cb = 0;
   bool fock = false;  // the vector is in the occupation basis (operators at equal times)
+  // Small blocks (a row per lane, at most 12): the row of the next operator's matrix and its eigenvalue are
+  // loaded as soon as the current row is used, and the weights are formed beside the products, so that
+  // the chain from one vector to the next holds neither a load nor an exponential. The next G operators'
+  // times and flavors are read one turn ahead. 16 steps of 1,024 five-orbital chains 2,660 -> 2,390 us
+  // (cached 2,738 -> 2,300), 777 five-orbital ratios 77 -> 61, 4,096 in FP64 457 -> 376 us. It wants 128
+  // registers: with a warp per walker four CTAs of four warps per SM, where five at 96 registers (spills)
+  // take 429 us for the FP64 ratios and seven without the read-ahead 453.
+  constexpr bool PRE = R == 1 && NV <= 6;
+  float4 row[PRE ? NV : 1];
+  E lam = eig_zero<MODE>();
+  if constexpr (PRE)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) row[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto fetch = [&](int mo, int pj) {
+    const int ds = (pj >> 16) & 63, dd = (pj >> 22) & 63, nv = (ds + T::EPV - 1) / T::EPV;
+    if (gl < dd) {
+      const float4 *p = (const float4 *)M.eig_mat + (size_t)mo + gl * nv;
+#pragma unroll
+      for (int v = 0; v < (PRE ? NV : 1); ++v)
+        if (v < nv) row[v] = __ldg(p + v);
+      lam = eig_lambda<MODE>(M, (pj & 0xffff) + gl);
+    }
+  };
+  Op op_next{0.0, 0, 0};
+  double t_next = 0.0;
+  auto fetch_ops = [&](int s) {
+    if (s < n) {
+      const int idx = half ? wk.i0 - s : wk.i0 + s;
+      op_next = cur.get(idx);
+      t_next = s + 1 == n ? wk.t_end : cur.get(half ? idx - 1 : idx + 1).t;
+    }
+  };
+  if constexpr (PRE) fetch_ops(gl);
   double Ll = 0.0;  // per lane: its operators' share of the log-weight; CACHED: the group's sum so far
   for (int base = 0; base < nmax; base += G) {
     // the next G operators of the half, one per lane
-    const int s = base + gl, idx = half ? wk.i0 - s : wk.i0 + s;
+    const int s = base + gl;
     const bool have = s < n;
+    if constexpr (!PRE) fetch_ops(s);
     int moff = 0, pk = 0, tgt = 0, code = 0;
     EigDt dt{0.f, 0.f, 0.0};
     if (have) {
-      const Op op = cur.get(idx);
-      const double tn = s + 1 == n ? wk.t_end : cur.get(half ? idx - 1 : idx + 1).t;
-      dt.d = half ? op.t - tn : tn - op.t;
-      code = 2 * op.f + (half ? 1 - op.dag : op.dag);
+      dt.d = half ? op_next.t - t_next : t_next - op_next.t;
+      code = 2 * op_next.f + (half ? 1 - op_next.dag : op_next.dag);
     }
+    if constexpr (PRE) fetch_ops(s + G);
     const int dn = have ? key_step(code) : 0, dm = have ? (1 << (code >> 2)) & M.key_mask : 0;
     int pn = dn, pm = dm;
     key_scan<G>(pn, pm, gl);
@@ -530,6 +588,10 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
       Ll += Lop;
     }
     const int cnt = min(G, nmax - base);
+    int Ej = 0;  // CACHED: the power of two and the shift when this lane's operator was done
+    double Lj = 0.0;
+    bool vj = false;
+    if constexpr (PRE) fetch(__shfl_sync(FULL, moff, 0, G), __shfl_sync(FULL, pk, 0, G));
     for (int j = 0; j < cnt; ++j) {
       if (BUILD && j >= dead) u.vanished = true;
       const bool act = base + j < n && !(BUILD && u.vanished);
@@ -542,27 +604,52 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
         dj.l = __shfl_sync(FULL, dt.l, j, G);
       }
       const int eoff = pj & 0xffff, ds = (pj >> 16) & 63, dd = (pj >> 22) & 63;
-      const int nv = (ds + T::EPV - 1) / T::EPV;
       const float4 *xv = reinterpret_cast<const float4 *>(xs + cb * DP);
-      E acc[R];
+      E acc[R], wt[R];
+      if constexpr (PRE) {
+        wt[0] = eig_weight<MODE>(M, lam, dj);
+        if constexpr (MODE == EIG_PAIR) {
+          // vectors past the source's rows meet zeros of xs; the second half is left out where neither
+          // group of the warp needs it
+          float a[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int i = 0; i < R; ++i) {
-        acc[i] = eig_zero<MODE>();
-        const int r = gl + G * i;
-        if (r < dd) {
-          const float4 *row = (const float4 *)M.eig_mat + (size_t)mo + r * nv;
-          if constexpr (NV <= 6) {
+          for (int v = 0; v < NV / 2; ++v) eig_fma4(a, row[v], xv[v]);
+          if (__any_sync(FULL, ds > NV / 2 * T::EPV))
 #pragma unroll
-            for (int v = 0; v < NV; ++v)
-              if (v < nv) eig_fma<MODE>(acc[i], __ldg(row + v), xv[v]);
-          } else {
+            for (int v = NV / 2; v < NV; ++v) eig_fma4(a, row[v], xv[v]);
+          float h, l;
+          eig_two_sum(a[0], (a[1] + a[2]) + a[3], h, l);
+          acc[0] = make_float2(h, l);
+        } else {
+          acc[0] = eig_zero<MODE>();
+          const int nv = (ds + T::EPV - 1) / T::EPV;
+#pragma unroll
+          for (int v = 0; v < NV; ++v)
+            if (v < nv) eig_fma<MODE>(acc[0], row[v], xv[v]);
+        }
+        if (gl >= dd) acc[0] = eig_zero<MODE>();
+        if (j + 1 < cnt) fetch(__shfl_sync(FULL, moff, j + 1, G), __shfl_sync(FULL, pk, j + 1, G));
+      } else {
+        const int nv = (ds + T::EPV - 1) / T::EPV;
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          acc[i] = eig_zero<MODE>();
+          const int r = gl + G * i;
+          if (r < dd) {
+            const float4 *p = (const float4 *)M.eig_mat + (size_t)mo + r * nv;
+            if constexpr (NV <= 6) {
+#pragma unroll
+              for (int v = 0; v < NV; ++v)
+                if (v < nv) eig_fma<MODE>(acc[i], __ldg(p + v), xv[v]);
+            } else {
 #pragma unroll 6
-            for (int v = 0; v < nv; ++v) eig_fma<MODE>(acc[i], __ldg(row + v), xv[v]);
-          }
-          if constexpr (MODE == EIG_PAIR) {
-            float h, l;
-            eig_two_sum(acc[i].x, acc[i].y, h, l);
-            acc[i] = make_float2(h, l);
+              for (int v = 0; v < nv; ++v) eig_fma<MODE>(acc[i], __ldg(p + v), xv[v]);
+            }
+            if constexpr (MODE == EIG_PAIR) {
+              float h, l;
+              eig_two_sum(acc[i].x, acc[i].y, h, l);
+              acc[i] = make_float2(h, l);
+            }
           }
         }
       }
@@ -605,13 +692,16 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
             }
           }
         if (gl == j) {
-          double2 *lg = half ? (out ? C.blog : C.sblog) : (out ? C.flog : C.sflog);
-          int32_t *bk = half ? (out ? C.bblk : C.sbblk) : (out ? C.fblk : C.sfblk);
-          bk[e] = u.vanished ? -1 : tgt;
-          lg[e] = make_double2(u.vanished ? 0.0 : L0 + Lpre + Lx + (double)ex * 0.69314718055994530942, 1.0);
+          Ej = ex;
+          Lj = Lx;
+          vj = u.vanished;
         }
       }
-      if (!eig_interval<MODE, G, R>(M, u.x, act && !u.vanished && !fock, gl, eoff, dd, dj, Lx, ex, sc)) u.vanished = true;
+      if constexpr (!PRE)
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+          wt[i] = gl + G * i < dd ? eig_weight<MODE>(M, eig_lambda<MODE>(M, eoff + gl + G * i), dj) : eig_zero<MODE>();
+      if (!eig_interval<MODE, G, R>(M, u.x, wt, act && !u.vanished && !fock, gl, eoff, dd, dj, Lx, ex, sc)) u.vanished = true;
       cb ^= 1;
 #pragma unroll
       for (int i = 0; i < R; ++i) {
@@ -620,6 +710,17 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
       }
       __syncwarp();
       if (act) u.dim = dd;
+    }
+    if (CACHED && wk.store && have) {
+      // log-weights and blocks of the states stored in this turn, all lanes at once: four FP64
+      // instructions for G states, where one lane per operator spent them on every operator
+      const int ij = half ? wk.i0 - s : wk.i0 + s;
+      const bool out = half ? ij >= wk.hi : ij + 1 <= wk.lo;
+      const size_t e = wk.eb + (half ? Kn - ij : ij + 1);
+      double2 *lg = half ? (out ? C.blog : C.sblog) : (out ? C.flog : C.sflog);
+      int32_t *bk = half ? (out ? C.bblk : C.sbblk) : (out ? C.fblk : C.sfblk);
+      bk[e] = vj ? -1 : tgt;
+      lg[e] = make_double2(vj ? 0.0 : L0 + Lpre + Lj + (double)Ej * 0.69314718055994530942, 1.0);
     }
     const int last = min(n - base, G) - 1;  // the block after the group's last operator so far
     const int tl = __shfl_sync(FULL, tgt, max(last, 0), G);
@@ -867,7 +968,7 @@ __device__ __forceinline__ void eig_output(const DevModel &M, int w, int has_mov
 constexpr int EIG_PLAIN = 0, EIG_RATIO = 1, EIG_BUILD = 2, EIG_MEASURE = 3;
 
 template <int MODE, int G, int DMAX, bool MEAS, int CACHE, bool SOLO>
-__global__ void __launch_bounds__(SOLO ? 128 : 256, SOLO ? (DMAX <= 10 && G == 16 ? 7 : 4) : 2)
+__global__ void __launch_bounds__(SOLO ? 128 : 256, SOLO ? 4 : 2)
     eig_kernel(DevModel M, SeqView S, MoveView mv, int has_moves, const int8_t *cur_sign, const double *cur_logabs,
                Workspace ws, CacheView C, int write, int8_t *sign, double *logv, int32_t *status, double *obs) {
   using H = EigHalf<MODE, G, DMAX>;
