@@ -433,12 +433,12 @@ template <int EPI>
 int gemm_tiles(const void *A, int lda, const void *B, int ldb, const mlp::Epi &epi, int M, int N, int K, int *err,
                cudaStream_t st, int splits = 1) {
   // column tile: the whole N when it fits the accumulator, narrower (128, then 64 columns)
-  // while the grid would have fewer than 64 CTAs, so that small batches still spread out
+  // while the grid would have fewer than 128 CTAs, so that small batches still spread out
   const int gm = (M + mlp::BM - 1) / mlp::BM, gz = gemm_splits(K, splits);
   int BN = N <= mlp::MAX_BN ? N : 128;
   if (EPI != mlp::EPI_OUT)  // whole rows in one tile
     for (const int w : {128, 64})
-      if (BN > w && gm * ((N + BN - 1) / BN) * gz < 64) BN = w;
+      if (BN > w && gm * ((N + BN - 1) / BN) * gz < 128) BN = w;
   // every slice holds at least one 64-column chunk of K (its offset keeps rows 16-byte aligned)
   const int kslice = ((K + splits - 1) / splits + mlp::BK - 1) / mlp::BK * mlp::BK;
   const dim3 grid((unsigned)gm, (unsigned)((N + BN - 1) / BN), (unsigned)((K + kslice - 1) / kslice));
