@@ -843,37 +843,38 @@ __global__ void sweep_record_kernel(SweepView S, __nv_bfloat16 *feat, float *tar
   if (lane == 0) targ[slot] = (float)(S.p_kind[w] == 0 ? S.r_log[w] : -S.r_log[w]);
 }
 
-// wt: per-walker weight of the measurement (NULL: 1), the Metropolis steps the walker spends
-// in the measured configuration in multi-try delayed acceptance
+// One warp per walker and flavor. wt: per-walker weight of the measurement (NULL: 1), the Metropolis steps
+// the walker spends in the measured configuration in multi-try delayed acceptance. A warp that took
+// a walker's flavors in turn waited for each flavor's loads and divisions: 1,024 chains of ten
+// flavors 46 -> 38 us; the FP64 pipe (18 instructions for 32 pairs) bounds it at 20.
 __global__ void sweep_measure_kernel(SweepView S, const int32_t *__restrict__ wt) {
   const int lane = threadIdx.x & 31;
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= S.nw) return;
+  const long long id = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (id >= (long long)S.nw * S.nf) return;
+  const int w = (int)(id / S.nf), f = (int)(id - (long long)w * S.nf);
   const double s = (double)S.w_sign[w] * (wt ? (double)wt[w] : 1.0);
-  const int nf = S.nf, kc = S.kcap, nb = S.n_bins;
+  const int kc = S.kcap, nb = S.n_bins;
   const double beta = S.beta;
+  const size_t fb = (size_t)id;
+  const int k = S.kf[fb];
   if (lane == 0) {
-    S.sign_sum[w] += s;
-    if (w == 0) atomicAdd(&S.counters[C_MEAS], 1ull);
+    if (f == 0) S.sign_sum[w] += s;
+    if (id == 0) atomicAdd(&S.counters[C_MEAS], 1ull);
+    S.order_sum[fb] += s * k;
   }
-  for (int f = 0; f < nf; ++f) {
-    const size_t fb = (size_t)w * nf + f;
-    const int k = S.kf[fb];
-    if (lane == 0) S.order_sum[fb] += s * k;
-    const double *Mf = S.M + fb * kc * kc;
-    const double *rt = S.row_t + fb * kc, *ct = S.col_t + fb * kc;
-    double *g = S.g_acc + fb * nb;
-    for (int e = lane; e < k * k; e += 32) {
-      const int j = e / k, i = e - j * k;
-      double x = ct[j] - rt[i], v = Mf[(size_t)j * kc + i];
-      if (x < 0.0) {
-        x += beta;
-        v = -v;
-      }
-      int b = (int)(x / beta * nb);
-      b = b > nb - 1 ? nb - 1 : (b < 0 ? 0 : b);
-      atomicAdd(g + b, s * v);
+  const double *Mf = S.M + fb * kc * kc;
+  const double *rt = S.row_t + fb * kc, *ct = S.col_t + fb * kc;
+  double *g = S.g_acc + fb * nb;
+  for (int e = lane; e < k * k; e += 32) {
+    const int j = e / k, i = e - j * k;
+    double x = ct[j] - rt[i], v = Mf[(size_t)j * kc + i];
+    if (x < 0.0) {
+      x += beta;
+      v = -v;
     }
+    int b = (int)(x / beta * nb);
+    b = b > nb - 1 ? nb - 1 : (b < 0 ? 0 : b);
+    atomicAdd(g + b, s * v);
   }
 }
 
@@ -1483,7 +1484,7 @@ static kt_status run_steps(kt_sweep *s, int32_t n_steps, const double *uniforms,
       kt::launch_cache_commit(s->cache, v.nw, M.n_kept, w.desc, w.wstatus, v.p_acc, v.r_status, s->cache_words, st);
     }
     if (meas_every > 0 && (step + 1) % meas_every == 0) {
-      kt::sweep_measure_kernel<<<grid, wpb * 32, 0, st>>>(v, nullptr);
+      kt::sweep_measure_kernel<<<(unsigned)(((long long)v.nw * v.nf + 7) / 8), 256, 0, st>>>(v, nullptr);
       if (s->measure_obs) {
         if (current_traces(s, v.m_sign, v.m_log, v.m_status, v.obs_tmp, st) != 0) return KT_ECUDA;
         const int n = v.nw * v.nobs;
@@ -1537,7 +1538,7 @@ kt_status kt_sweep_run_da_multi(kt_sweep *s, int32_t n_steps, int32_t tries, con
     kt::sweep_select_kernel<<<grid, wpb * 32, 0, st>>>(v, tv, u);
     // measurement of the configuration the walker spent this step's tries in, weighted by them
     if (meas_every > 0 && (step + 1) % meas_every == 0) {
-      kt::sweep_measure_kernel<<<grid, wpb * 32, 0, st>>>(v, tv.n_tries);
+      kt::sweep_measure_kernel<<<(unsigned)(((long long)v.nw * v.nf + 7) / 8), 256, 0, st>>>(v, tv.n_tries);
       if (s->measure_obs) {
         if (current_traces(s, v.m_sign, v.m_log, v.m_status, v.obs_tmp, st) != 0) return KT_ECUDA;
         const int n = v.nw * v.nobs;
