@@ -122,7 +122,7 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(rows)}
 
 
-ITEMS_SOURCES = ("kt_internal.h", "kt_device.cuh", "kt_items.cuh", "kt_items_f32.cu")
+ITEMS_SOURCES = ("kt_internal.h", "kt_device.cuh", "kt_eig.cuh", "kt_eig_f32.cu")
 
 
 def trim_hist(h):
@@ -132,7 +132,7 @@ def trim_hist(h):
 
 
 def source_sha() -> str:
-    """Hash of the sources the FP32 Krylov items kernel is compiled from (ties the committed
+    """Hash of the sources the FP32 kernel of a ratio call is compiled from (ties the committed
     ncu traffic record of that kernel to its code)."""
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_0908_0681_gb300", "csrc")
@@ -142,8 +142,19 @@ def source_sha() -> str:
     return h.hexdigest()[:16]
 
 
+def mean_block_square(n_orb: int) -> float:
+    """Mean squared size of the invariant blocks (n_up, n_dn, singly occupied orbitals)."""
+    import numpy as np
+
+    x = np.arange(4 ** n_orb)
+    up, dn = [(x >> 2 * a) & 1 for a in range(n_orb)], [(x >> 2 * a + 1) & 1 for a in range(n_orb)]
+    mask = sum((up[a] ^ dn[a]) << a for a in range(n_orb))
+    d = np.unique((sum(up) * (n_orb + 1) + sum(dn)) * 2 ** n_orb + mask, return_counts=True)[1]
+    return float((d * d).sum()) / len(d)
+
+
 def measured_traffic(sha: str):
-    """dram read+write bytes per items-kernel launch from a committed ncu summary, if it
+    """dram read+write bytes per launch of that kernel from a committed ncu summary, if it
     was taken on the current kernel source; else None."""
     p = os.path.join(ROOT, "profiles", "items_kernel_traffic.json")
     try:
@@ -1039,20 +1050,20 @@ def main():
                             "weights, FP64 QL where Ritz values are too close)"}
     e2e_value = world * n / (e2e_ms / 1000.0)
 
-    # roofline of the dominant kernel (Krylov items)
+    # roofline of the kernel of a ratio call (block eigenbasis)
     items_ms = stage32["items"] / max(nl32, 1)
     sha = source_sha()
     mhz = clocks.get("sm_max_mhz") or 2070.0
     peak32 = SM_COUNT_GB300 * FP32_LANES_PER_SM * 2 * mhz * 1e6 / 1e12
     peak64 = SM_COUNT_GB300 * FP64_FMA_PER_SM_CLK * 2 * mhz * 1e6 / 1e12
-    f32_per_launch = st["flops_alg"] / a.steps
+    f32_per_launch = st["intervals"] / a.steps * 2 * mean_block_square(w.model.n_orb)
     ach32 = f32_per_launch / (items_ms / 1000.0) / 1e12
-    # The algorithmic work of the path is the Krylov vector arithmetic on the FP32 pipe;
-    # its serial per-walker dependency chain (not a pipe) is what bounds the kernel.
+    # The algorithmic work of the path is one dense block-to-block product per interval on the FP32
+    # pipe; its serial per-walker dependency chain (not a pipe) is what bounds the kernel.
     roofline = {"bound": "alu", "achieved": ach32, "peak": peak32, "unit": "TFLOP/s", "frac": ach32 / peak32,
-                "traffic": measured_traffic(sha), "kernel": "items_kernel", "pipe": "fp32",
+                "traffic": measured_traffic(sha), "kernel": "eig_kernel", "pipe": "fp32",
                 "flops_per_launch": f32_per_launch,
-                "flops_definition": "sum over Krylov intervals of p (2 nnz(H_b) + 11 d_b) + 2 p d_b (kt_stats.flops_alg)",
+                "flops_definition": "propagated intervals (kt_stats.intervals) times 2 d^2, the mean over the blocks",
                 "reorth_flops_per_launch": st["flops_reorth"] / a.steps,
                 "device_flops_vec_per_launch": st["flops_vec"] / a.steps,
                 "items_ms_per_launch": items_ms,
@@ -1092,7 +1103,7 @@ def main():
             "config": {"workload": f"{a.workload}_{n}_walkers" + ("" if a.trunc_eps is None else f"_trunc{a.trunc_eps:g}"), "n_orb": w.model.n_orb, "U": w.model.U,
                        "J": w.model.J, "beta": w.model.beta,
                        "walkers_per_gpu": n, "mean_ops_per_walker": float(seqs.offsets[-1]) / n,
-                       "krylov_tol": w.model.krylov_tol, "trunc_eps": w.model.trunc_eps, "precision": "fp32-krylov (double-float tridiagonal scalars and norms, fp64 log-weights)",
+                       "krylov_tol": w.model.krylov_tol, "trunc_eps": w.model.trunc_eps, "precision": "fp32 pairs in the block eigenbasis (exact leading products, fp64 log-weights)",
                        "blocks": "(n_up, n_dn, singly-occupied mask)", "n_blocks": info["n_blocks"],
                        "d_max": info["d_max"], "n_kept": info["n_kept"], "group_lanes": tuned, "l2": "flushed (256 MiB write) before every timed step",
                        "parallelism": f"replicas x{world}"},
@@ -1115,8 +1126,8 @@ def main():
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
             "sweep": sweep,
             "clocks": clocks,
-            # prep, prune, order, items and reduce per ratio call
-            "gpu_launches": 5 * a.steps,
+            # one kernel per ratio call (traces in the block eigenbasis)
+            "gpu_launches": a.steps,
             "kernel_source_sha": sha,
         }
         print(json.dumps(line), flush=True)
