@@ -259,6 +259,25 @@ __global__ void measure_plan_kernel(DevModel M, SeqView S, Workspace ws, CacheVi
   }
 }
 
+// n words by one warp, eight loads a lane in flight: a loop that stores each word before it loads the
+// next waits for every load (1,024 chains, 17 us a step before).
+__device__ __forceinline__ void copy_words(const uint32_t *src, uint32_t *dst, int n, int lane) {
+  for (int base = 0; base < n; base += 256) {
+    uint32_t t[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int k = base + 32 * c + lane;
+      t[c] = k < n ? src[k] : 0u;
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int k = base + 32 * c + lane;
+      if (k < n) dst[k] = t[c];
+    }
+  }
+}
+
+
 // After the accept decision of a cached step, one warp per (walker, kept state)
 // item: an accepted move makes its tentative states (scratch) the cache's and the
 // valid ranges meet at m; a rejected one keeps the cache and only extends the valid
@@ -301,26 +320,30 @@ __global__ void cache_commit_kernel(CacheView C, int n, int nk, const int4 *__re
     return;
   }
   const size_t eb = (size_t)item * ((size_t)C.P + 1);
-  const uint32_t *sfv = (const uint32_t *)C.sfvec, *sbv = (const uint32_t *)C.sbvec;
-  uint32_t *fv = (uint32_t *)C.fvec, *bv = (uint32_t *)C.bvec;
   // forward slots (max(y, lo), m] and backward reverse slots of positions [m, min(x, hi))
   const int f0 = max(y, lo) + 1, nfw = m - f0 + 1;
   const int r0 = Kn - min(x, hi) + 1, nbw = (Kn - m) - r0 + 1;
-  for (int k = lane; k < nfw * words; k += 32) {
-    const size_t e = eb + f0 + k / words;
-    fv[e * words + k % words] = sfv[e * words + k % words];
-  }
-  for (int k = lane; k < nbw * words; k += 32) {
-    const size_t e = eb + r0 + k / words;
-    bv[e * words + k % words] = sbv[e * words + k % words];
-  }
-  for (int k = lane; k < nfw; k += 32) {
-    C.fblk[eb + f0 + k] = C.sfblk[eb + f0 + k];
-    C.flog[eb + f0 + k] = C.sflog[eb + f0 + k];
-  }
-  for (int k = lane; k < nbw; k += 32) {
-    C.bblk[eb + r0 + k] = C.sbblk[eb + r0 + k];
-    C.blog[eb + r0 + k] = C.sblog[eb + r0 + k];
+  copy_words((const uint32_t *)C.sfvec + (eb + f0) * words, (uint32_t *)C.fvec + (eb + f0) * words, nfw * words, lane);
+  copy_words((const uint32_t *)C.sbvec + (eb + r0) * words, (uint32_t *)C.bvec + (eb + r0) * words, nbw * words, lane);
+  for (int k = lane; k < max(nfw, nbw); k += 32) {
+    int32_t bf = 0, bb = 0;
+    double2 lf = make_double2(0.0, 0.0), lb = lf;
+    if (k < nfw) {
+      bf = C.sfblk[eb + f0 + k];
+      lf = C.sflog[eb + f0 + k];
+    }
+    if (k < nbw) {
+      bb = C.sbblk[eb + r0 + k];
+      lb = C.sblog[eb + r0 + k];
+    }
+    if (k < nfw) {
+      C.fblk[eb + f0 + k] = bf;
+      C.flog[eb + f0 + k] = lf;
+    }
+    if (k < nbw) {
+      C.bblk[eb + r0 + k] = bb;
+      C.blog[eb + r0 + k] = lb;
+    }
   }
   if (lane == 0) {
     C.f[item] = m;
