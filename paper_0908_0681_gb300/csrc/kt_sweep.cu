@@ -421,38 +421,65 @@ __device__ __forceinline__ void accept_walker(const SweepView &S, double u5, con
     const double tA = td < ta ? td : ta, tB = td < ta ? ta : td;
     const int dA = td < ta ? 1 : 0, dB = 1 - dA;
     // new index i: i < p1 old i; i == p1 A; p1 < i <= p2 old i-1; i == p2+1 B; else old i-2.
-    // Chunks from the top: every source index is <= i, read before any write of the chunk.
+    // 128 operators at a time from the top: every source index is <= i, read before any write of the chunk.
     const int Kn = d.w;
-    for (int top = Kn - 1; top >= 0; top -= 32) {
-      const int i = top - lane;
-      double t = 0.0;
-      int g = 0, h = 0;
-      if (i >= 0) {
-        int src = -1;
-        if (i < d.y) src = i;
-        else if (i == d.y) { t = tA; g = f; h = dA; }
-        else if (i <= d.z) src = i - 1;
-        else if (i == d.z + 1) { t = tB; g = f; h = dB; }
-        else src = i - 2;
-        if (src >= 0) { t = tau[src]; g = fl[src]; h = dg[src]; }
+    for (int top = Kn - 1; top >= 0; top -= 128) {
+      double t[4];
+      int g[4], h[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int i = top - 32 * c - lane;
+        const bool a = i == d.y, b = i == d.z + 1;
+        const int src = i < d.y ? i : (i <= d.z ? i - 1 : i - 2);
+        t[c] = a ? tA : tB;
+        g[c] = f;
+        h[c] = a ? dA : dB;
+        if (i >= 0 && !a && !b) {
+          t[c] = tau[src];
+          g[c] = fl[src];
+          h[c] = dg[src];
+        }
       }
       __syncwarp();
-      if (i >= 0) { tau[i] = t; fl[i] = (uint8_t)g; dg[i] = (uint8_t)h; }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int i = top - 32 * c - lane;
+        if (i >= 0) {
+          tau[i] = t[c];
+          fl[i] = (uint8_t)g[c];
+          dg[i] = (uint8_t)h[c];
+        }
+      }
       __syncwarp();
     }
   } else {
-    // new index i: i < p1 old i; p1 <= i < p2 - 1 old i+1; else old i+2. Chunks from the bottom.
+    // new index i: i < p1 old i; p1 <= i < p2 - 1 old i+1; else old i+2. From the bottom.
     const int Kn = d.w;
-    for (int base = 0; base < Kn; base += 32) {
-      const int i = base + lane;
-      double t = 0.0;
-      int g = 0, h = 0;
-      if (i < Kn) {
+    for (int base = 0; base < Kn; base += 128) {
+      double t[4];
+      int g[4], h[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int i = base + 32 * c + lane;
         const int src = i < d.y ? i : (i < d.z - 1 ? i + 1 : i + 2);
-        t = tau[src]; g = fl[src]; h = dg[src];
+        t[c] = 0.0;
+        g[c] = h[c] = 0;
+        if (i < Kn) {
+          t[c] = tau[src];
+          g[c] = fl[src];
+          h[c] = dg[src];
+        }
       }
       __syncwarp();
-      if (i < Kn) { tau[i] = t; fl[i] = (uint8_t)g; dg[i] = (uint8_t)h; }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int i = base + 32 * c + lane;
+        if (i < Kn) {
+          tau[i] = t[c];
+          fl[i] = (uint8_t)g[c];
+          dg[i] = (uint8_t)h[c];
+        }
+      }
       __syncwarp();
     }
   }
