@@ -100,8 +100,7 @@ __device__ __forceinline__ void stage_tile(uint8_t *dst, const __nv_bfloat16 *sr
 //   EPI_STORE  C = acc
 //   EPI_ACT1   H1 = bf16(relu(acc + bias)), with C the FP32 acc too, with hT the transpose too
 //   EPI_OUT    y = v . relu(acc + bias) + *vb, for tiles that hold whole rows (N = 256 = BN)
-//   EPI_DZ1    C = acc (dH1), hT = transpose of bf16(acc masked by Z + bias > 0), part = column sums of
-//              the masked FP32 values per 32 rows
+//   EPI_DZ1    C = acc (dH1), hT = transpose of bf16(acc masked by Z + bias > 0)
 enum { EPI_STORE, EPI_ACT1, EPI_OUT, EPI_DZ1 };
 struct Epi {
   float *C;
@@ -109,16 +108,14 @@ struct Epi {
   const float *bias;
   __nv_bfloat16 *h, *hT;  // [M][ldc], [N][M]
   const float *Z;         // [M][ldc]
-  float *part;            // [ceil(M / 32)][ldc]
   const float *v, *vb;
   float *y;
 };
 
-// Warp w holds rows m0 + 32w .. (one per lane); 32 accumulator columns at a time. `tile`: 4 x 32 x 33
-// floats of shared memory (EPI_DZ1). A lane writes 16 bytes at a time where C allows it, transposes
-// are written by 32 consecutive rows.
+// Warp w holds rows m0 + 32w .. (one per lane); 32 accumulator columns at a time. A lane writes 16 bytes
+// at a time where C allows it, transposes are written by 32 consecutive rows.
 template <int EPI>
-__device__ __forceinline__ void tile_epilogue(uint32_t tmem, int m0, int n0, int bn, int M, const Epi &e, float *tile) {
+__device__ __forceinline__ void tile_epilogue(uint32_t tmem, int m0, int n0, int bn, int M, const Epi &e) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, row = m0 + warp * 32 + lane;
   const bool vec = (e.ldc & 3) == 0 && ((uintptr_t)e.C & 15) == 0;
   float acc[EPI == EPI_OUT ? 32 : 1];
@@ -176,26 +173,20 @@ __device__ __forceinline__ void tile_epilogue(uint32_t tmem, int m0, int n0, int
       for (int j = 0; j < 32; ++j)
         acc[j] = fmaf(fmaxf(__uint_as_float(r[j]) + __ldg(e.bias + n + j), 0.f), __ldg(e.v + n + j), acc[j]);
     } else if constexpr (EPI == EPI_DZ1) {
-      float *t = tile + warp * 32 * 33;
-      const float4 *z = reinterpret_cast<const float4 *>(e.Z + (size_t)row * e.ldc + n);
+      if (row < M) {
+        const float4 *z = reinterpret_cast<const float4 *>(e.Z + (size_t)row * e.ldc + n);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float4 zq = row < M ? z[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float zz[4] = {zq.x, zq.y, zq.z, zq.w};
+        for (int q = 0; q < 8; ++q) {
+          const float4 zq = z[q];
+          const float zz[4] = {zq.x, zq.y, zq.z, zq.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int j = 4 * q + i;
-          const float d = row < M && zz[i] + __ldg(e.bias + n + j) > 0.f ? __uint_as_float(r[j]) : 0.f;
-          if (row < M) e.hT[(size_t)(n + j) * M + row] = __float2bfloat16_rn(d);
-          t[lane * 33 + j] = d;
+          for (int i = 0; i < 4; ++i) {
+            const int j = 4 * q + i;
+            const float d = zz[i] + __ldg(e.bias + n + j) > 0.f ? __uint_as_float(r[j]) : 0.f;
+            e.hT[(size_t)(n + j) * M + row] = __float2bfloat16_rn(d);
+          }
         }
       }
-      __syncwarp();
-      float sum = 0.f;
-#pragma unroll 8
-      for (int i = 0; i < 32; ++i) sum += t[i * 33 + lane];
-      if (m0 + warp * 32 < M) e.part[(size_t)((m0 >> 5) + warp) * e.ldc + n + lane] = sum;
-      __syncwarp();
     }
   }
   if constexpr (EPI == EPI_OUT) {
@@ -283,7 +274,7 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __nv_bfloat16 *__r
     }
   }
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (!abort_sh) tile_epilogue<EPI>(tmem, m0, n0, bn, M, epi, reinterpret_cast<float *>(smem));
+  if (!abort_sh) tile_epilogue<EPI>(tmem, m0, n0, bn, M, epi);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
@@ -398,7 +389,7 @@ __global__ void __launch_bounds__(128) gemm_bf16_tma_kernel(const __grid_constan
   __syncwarp();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   __syncthreads();
-  if (!abort_sh) tile_epilogue<EPI>(tmem, m0, n0, bn, M, epi, reinterpret_cast<float *>(smem));
+  if (!abort_sh) tile_epilogue<EPI>(tmem, m0, n0, bn, M, epi);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
@@ -502,22 +493,22 @@ __global__ void transpose_bf16_kernel(const float *__restrict__ src, __nv_bfloat
 
 // Training, after z2: a block of 256 threads takes 32 rows (4 per warp, a lane every 32nd column) from
 // z2 to y, the loss, dy = 2 (y - t) / B and dZ2 = bf16(dy w3 masked by relu'(z2 + b2)) in both layouts,
-// and leaves its rows' sums of dy H2, of the unrounded dZ2 and of dy; Z2 is read once. The blocks from n_out
-// on transpose X in tiles of 64 x 64 for dW1, which has nothing to wait for. One launch for what were
-// six and a memset: every one of them ran 2 to 9 microseconds on a few megabytes from L2.
+// and leaves its rows' share of the loss. The blocks from n_out on transpose X in tiles of 64 x 64 for
+// dW1, which has nothing to wait for. One launch for what were four and a memset: every one of them ran 2
+// to 9 microseconds on a few megabytes from L2.
 constexpr int ROWS = 32, PITCH = ROWS + 2;
 struct OutTrain {
   const float *Z2, *b2, *w3, *b3, *t;
   float *y, *dy;
   __nv_bfloat16 *dZ2, *dZ2T;
-  float *pw3, *pb2, *pb3, *ploss;  // per block of rows
+  float *ploss;  // per block of rows
   const __nv_bfloat16 *X;
   __nv_bfloat16 *XT;
   int B, nin, n_out;
 };
 __global__ void __launch_bounds__(256) out_train_kernel(OutTrain A) {
   __shared__ __align__(16) __nv_bfloat16 tile[H * PITCH];
-  __shared__ float sw3[8][H], sb2[8][H], sdy[8], slo[8];
+  __shared__ float slo[8];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, B = A.B;
   if ((int)blockIdx.x >= A.n_out) {
     constexpr int P = 66;
@@ -546,12 +537,11 @@ __global__ void __launch_bounds__(256) out_train_kernel(OutTrain A) {
     return;
   }
   const int r0 = blockIdx.x * ROWS, rows = min(ROWS, B - r0);
-  float b2[8], w3[8], a[8], s[8], sd = 0.f, lo = 0.f;
+  float b2[8], w3[8], lo = 0.f;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     b2[k] = __ldg(A.b2 + lane + 32 * k);
     w3[k] = __ldg(A.w3 + lane + 32 * k);
-    a[k] = s[k] = 0.f;
   }
   const float b3 = __ldg(A.b3);
 #pragma unroll
@@ -571,7 +561,6 @@ __global__ void __launch_bounds__(256) out_train_kernel(OutTrain A) {
       A.y[row] = y;
       A.dy[row] = d;
     }
-    sd += d;
     lo += e * e / (float)B;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -579,35 +568,13 @@ __global__ void __launch_bounds__(256) out_train_kernel(OutTrain A) {
       const __nv_bfloat16 v = __float2bfloat16_rn(z[k] > 0.f ? d * w3[k] : 0.f);
       A.dZ2[(size_t)row * H + j] = v;
       tile[j * PITCH + rr] = v;
-      a[k] = fmaf(d, fmaxf(z[k], 0.f), a[k]);
-      if (z[k] > 0.f) s[k] = fmaf(d, w3[k], s[k]);
     }
   }
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    sw3[warp][lane + 32 * k] = a[k];
-    sb2[warp][lane + 32 * k] = s[k];
-  }
-  if (lane == 0) {
-    sdy[warp] = sd;
-    slo[warp] = lo;
-  }
+  if (lane == 0) slo[warp] = lo;
   __syncthreads();
-  float x = 0.f, u = 0.f;
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    x += sw3[q][tid];
-    u += sb2[q][tid];
-  }
-  A.pw3[(size_t)blockIdx.x * H + tid] = x;
-  A.pb2[(size_t)blockIdx.x * H + tid] = u;
   if (tid == 0) {
-    float p = 0.f, l = 0.f;
-    for (int q = 0; q < 8; ++q) {
-      p += sdy[q];
-      l += slo[q];
-    }
-    A.pb3[blockIdx.x] = p;
+    float l = 0.f;
+    for (int q = 0; q < 8; ++q) l += slo[q];
     A.ploss[blockIdx.x] = l;
   }
   // the transpose: 16 bytes (8 rows) per lane, four lanes per column
@@ -619,8 +586,66 @@ __global__ void __launch_bounds__(256) out_train_kernel(OutTrain A) {
   }
 }
 
+// Column sums over the batch by chunks of CHUNK rows: dy H2 and the unrounded dZ2 (blockIdx.y 0, with the
+// sum of dy), the masked dH1 (1); 64 columns a block, 16 rows in flight. A column adds its chunk's rows one
+// by one and the chunks are added in order: that order is part of the results, since Adam's first steps turn
+// a gradient near zero into a full step of its sign (sums of 32 rows at a time moved weights by 2e-3).
+constexpr int CHUNK = 128;
+__global__ void __launch_bounds__(64) column_sums_kernel(const float *__restrict__ Z2, const float *__restrict__ b2,
+                                                         const float *__restrict__ w3, const float *__restrict__ dy,
+                                                         const float *__restrict__ dH1, const float *__restrict__ Z1,
+                                                         const float *__restrict__ b1, float *pw3, float *pb2, float *pb3,
+                                                         float *pb1, int B) {
+  __shared__ float sh[CHUNK];
+  const int c = blockIdx.x, t = threadIdx.x, j = blockIdx.z * 64 + t;
+  const int r0 = c * CHUNK, r1 = min(B, r0 + CHUNK);  // a multiple of 16 rows
+  if (blockIdx.y == 1) {
+    const float bj = b1[j];
+    float s = 0.f;
+    for (int b = r0; b < r1; b += 16) {
+      float z[16], d[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        z[i] = Z1[(size_t)(b + i) * H + j];
+        d[i] = dH1[(size_t)(b + i) * H + j];
+      }
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        if (z[i] + bj > 0.f) s += d[i];
+    }
+    pb1[(size_t)c * H + j] = s;
+    return;
+  }
+  const float bj = b2[j], wj = w3[j];
+  float a = 0.f, s = 0.f;
+  for (int b = r0; b < r1; b += 16) {
+    float z[16], d[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      z[i] = Z2[(size_t)(b + i) * H + j] + bj;
+      d[i] = dy[b + i];
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      a = fmaf(d[i], fmaxf(z[i], 0.f), a);
+      if (z[i] > 0.f) s = fmaf(d[i], wj, s);
+    }
+  }
+  pw3[(size_t)c * H + j] = a;
+  pb2[(size_t)c * H + j] = s;
+  if (blockIdx.z != 0) return;
+  sh[t] = r0 + t < r1 ? dy[r0 + t] : 0.f;
+  sh[t + 64] = r0 + t + 64 < r1 ? dy[r0 + t + 64] : 0.f;
+  __syncthreads();
+  for (int o = 64; o > 0; o >>= 1) {
+    if (t < o) sh[t] += sh[t + o];
+    __syncthreads();
+  }
+  if (t == 0) pb3[c] = sh[0];
+}
+
 // The gradients from their parts, one launch: the weight gradients' split-K slabs (in order), the
-// column sums of the blocks of rows (32 columns per block, 8 threads a column), db3 and the loss.
+// column sums of the chunks (in order, a thread per column), db3 and the loss.
 struct Grads {
   const float *part1, *part2;       // [S][H][nin], [S][H][H]
   float *gW1, *gW2;
@@ -628,10 +653,10 @@ struct Grads {
   float *gcol[3];                   // gw3, gb2, gb1
   const float *pb3, *ploss;
   float *gb3, *loss, *loss_out;
-  int S, nc, nin;
+  int S, nc, nb, nin;               // slabs, chunks, blocks of rows, inputs
 };
 __global__ void __launch_bounds__(256) grads_kernel(Grads G, int n1, int n2) {
-  __shared__ float sh[2][256];
+  __shared__ float sh[256];
   const int tid = threadIdx.x, blk = blockIdx.x;
   if (blk < n1 + n2) {
     const bool first = blk < n1;
@@ -652,38 +677,28 @@ __global__ void __launch_bounds__(256) grads_kernel(Grads G, int n1, int n2) {
     return;
   }
   const int c = blk - n1 - n2;
-  if (c < 3 * H / 32) {
-    const int k = c / (H / 32), j = c % (H / 32) * 32 + (tid & 31);
-    const float *p = k == 0 ? G.pcol[0] : (k == 1 ? G.pcol[1] : G.pcol[2]);
+  if (c < 3) {
+    const float *p = c == 0 ? G.pcol[0] : (c == 1 ? G.pcol[1] : G.pcol[2]);
     float s = 0.f;
-    for (int q = tid >> 5; q < G.nc; q += 8) s += p[(size_t)q * H + j];
-    sh[0][tid] = s;
-    __syncthreads();
-    if (tid < 32) {
-      for (int q = 1; q < 8; ++q) s += sh[0][tid + 32 * q];
-      (k == 0 ? G.gcol[0] : (k == 1 ? G.gcol[1] : G.gcol[2]))[j] = s;
-    }
+#pragma unroll 8
+    for (int q = 0; q < G.nc; ++q) s += p[(size_t)q * H + tid];
+    (c == 0 ? G.gcol[0] : (c == 1 ? G.gcol[1] : G.gcol[2]))[tid] = s;
     return;
   }
-  float a = 0.f, b = 0.f;
-  for (int q = tid; q < G.nc; q += 256) {
-    a += G.pb3[q];
-    b += G.ploss[q];
-  }
-  sh[0][tid] = a;
-  sh[1][tid] = b;
+  float b = 0.f;
+  for (int q = tid; q < G.nb; q += 256) b += G.ploss[q];
+  sh[tid] = b;
   __syncthreads();
   for (int o = 128; o > 0; o >>= 1) {
-    if (tid < o) {
-      sh[0][tid] += sh[0][tid + o];
-      sh[1][tid] += sh[1][tid + o];
-    }
+    if (tid < o) sh[tid] += sh[tid + o];
     __syncthreads();
   }
   if (tid == 0) {
-    G.gb3[0] = sh[0][0];
-    G.loss[0] = sh[1][0];
-    if (G.loss_out) G.loss_out[0] = sh[1][0];
+    float a = 0.f;
+    for (int q = 0; q < G.nc; ++q) a += G.pb3[q];
+    G.gb3[0] = a;
+    G.loss[0] = sh[0];
+    if (G.loss_out) G.loss_out[0] = sh[0];
   }
 }
 
@@ -727,7 +742,8 @@ struct kt_mlp {
   float *Z1, *Z2, *dH1, *y, *dy, *loss;
   __nv_bfloat16 *H1b, *H1Tb, *dZ2b, *dZ2Tb, *dZ1Tb, *XTb;
   float *part1, *part2;      // split-K slabs of the weight gradients
-  float *pw3, *pb2, *pb3, *pb1, *ploss;  // sums of 32 rows
+  float *pw3, *pb2, *pb3, *pb1;  // column sums of the chunks
+  float *ploss;              // by blocks of rows
   int *err;
 };
 
@@ -882,12 +898,14 @@ kt_status kt_mlp_backward(kt_mlp *n, const void *X, const float *t, int32_t B, f
   cudaStream_t st = (cudaStream_t)stream;
   const int nin = n->n_in;
   if (kt::mlp_forward(n, X, B, nullptr, true, st) != 0) return KT_ECUDA;
-  const int nc = (B + ROWS - 1) / ROWS, nt = (B + 63) / 64 * ((nin + 63) / 64);
-  out_train_kernel<<<nc + nt, 256, 0, st>>>(OutTrain{n->Z2, n->b2, n->w3, n->b3, t, n->y, n->dy, n->dZ2b, n->dZ2Tb, n->pw3,
-                                                     n->pb2, n->pb3, n->ploss, (const __nv_bfloat16 *)X, n->XTb, B, nin, nc});
-  // dH1 = dZ2 W2: A = dZ2 [B][H], B-operand = W2T [H(in)][H(out)]; its mask, dZ1 and db1 in the epilogue
-  Epi ed{n->dH1, H, n->b1, nullptr, n->dZ1Tb, n->Z1, n->pb1};
+  const int nb = (B + ROWS - 1) / ROWS, nc = (B + CHUNK - 1) / CHUNK, nt = (B + 63) / 64 * ((nin + 63) / 64);
+  out_train_kernel<<<nb + nt, 256, 0, st>>>(OutTrain{n->Z2, n->b2, n->w3, n->b3, t, n->y, n->dy, n->dZ2b, n->dZ2Tb, n->ploss,
+                                                     (const __nv_bfloat16 *)X, n->XTb, B, nin, nb});
+  // dH1 = dZ2 W2: A = dZ2 [B][H], B-operand = W2T [H(in)][H(out)]; its mask and dZ1 in the epilogue
+  Epi ed{n->dH1, H, n->b1, nullptr, n->dZ1Tb, n->Z1};
   if (kt::gemm_tiles<EPI_DZ1>(n->dZ2b, H, n->W2Tb, H, ed, B, H, H, n->err, st)) return KT_ECUDA;
+  column_sums_kernel<<<dim3((unsigned)nc, 2, H / 64), 64, 0, st>>>(n->Z2, n->b2, n->w3, n->dy, n->dH1, n->Z1, n->b1, n->pw3,
+                                                                   n->pb2, n->pb3, n->pb1, B);
   // weight gradients reduce over the batch: split K = B over several CTAs, the slabs summed below
   // dW2 = dZ2^T H1: A = dZ2T [H][B], B-operand = H1T [H][B]
   Epi e2{n->part2, H};
@@ -896,9 +914,9 @@ kt_status kt_mlp_backward(kt_mlp *n, const void *X, const float *t, int32_t B, f
   Epi e1{n->part1, nin};
   if (kt::gemm_tiles<EPI_STORE>(n->dZ1Tb, B, n->XTb, B, e1, H, nin, B, n->err, st, MAX_SPLITS)) return KT_ECUDA;
   const int n1 = (int)blocks((long long)H * nin / 4), n2 = (int)blocks((long long)H * H / 4);
-  grads_kernel<<<n1 + n2 + 3 * H / 32 + 1, 256, 0, st>>>(
+  grads_kernel<<<n1 + n2 + 4, 256, 0, st>>>(
       Grads{n->part1, n->part2, n->gW1, n->gW2, {n->pw3, n->pb2, n->pb1}, {n->gw3, n->gb2, n->gb1}, n->pb3, n->ploss,
-            n->gb3, n->loss, loss, kt::gemm_splits(B, MAX_SPLITS), nc, nin}, n1, n2);
+            n->gb3, n->loss, loss, kt::gemm_splits(B, MAX_SPLITS), nc, nb, nin}, n1, n2);
   n->lastB = B;
   return cudaGetLastError() == cudaSuccess ? KT_OK : KT_ECUDA;
 }
