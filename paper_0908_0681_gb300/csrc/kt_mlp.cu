@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(256) out_train_kernel(OutTrain A) {
 }
 
 // Column sums over the batch by chunks of CHUNK rows: dy H2 and the unrounded dZ2 (blockIdx.y 0, with the
-// sum of dy), the masked dH1 (1); 64 columns a block, 16 rows in flight. A column adds its chunk's rows one
+// sum of dy), the masked dH1 (1); 64 columns a block, 64 rows in flight. A column adds its chunk's rows one
 // by one and the chunks are added in order: that order is part of the results, since Adam's first steps turn
 // a gradient near zero into a full step of its sign (sums of 32 rows at a time moved weights by 2e-3).
 constexpr int CHUNK = 128;
@@ -602,15 +602,15 @@ __global__ void __launch_bounds__(64) column_sums_kernel(const float *__restrict
   if (blockIdx.y == 1) {
     const float bj = b1[j];
     float s = 0.f;
-    for (int b = r0; b < r1; b += 16) {
-      float z[16], d[16];
+    for (int b = r0; b < r1; b += 64) {
+      float z[64], d[64];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        z[i] = Z1[(size_t)(b + i) * H + j];
-        d[i] = dH1[(size_t)(b + i) * H + j];
+      for (int i = 0; i < 64; ++i) {
+        z[i] = b + i < r1 ? Z1[(size_t)(b + i) * H + j] : -INFINITY;
+        d[i] = b + i < r1 ? dH1[(size_t)(b + i) * H + j] : 0.f;
       }
 #pragma unroll
-      for (int i = 0; i < 16; ++i)
+      for (int i = 0; i < 64; ++i)
         if (z[i] + bj > 0.f) s += d[i];
     }
     pb1[(size_t)c * H + j] = s;
@@ -618,17 +618,18 @@ __global__ void __launch_bounds__(64) column_sums_kernel(const float *__restrict
   }
   const float bj = b2[j], wj = w3[j];
   float a = 0.f, s = 0.f;
-  for (int b = r0; b < r1; b += 16) {
-    float z[16], d[16];
+  for (int b = r0; b < r1; b += 64) {
+    float z[64], d[64];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      z[i] = Z2[(size_t)(b + i) * H + j] + bj;
-      d[i] = dy[b + i];
+    for (int i = 0; i < 64; ++i) {
+      z[i] = b + i < r1 ? Z2[(size_t)(b + i) * H + j] : -INFINITY;
+      d[i] = b + i < r1 ? dy[b + i] : 0.f;
     }
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      a = fmaf(d[i], fmaxf(z[i], 0.f), a);
-      if (z[i] > 0.f) s = fmaf(d[i], wj, s);
+    for (int i = 0; i < 64; ++i) {
+      const float v = z[i] + bj;
+      a = fmaf(d[i], fmaxf(v, 0.f), a);
+      if (v > 0.f) s = fmaf(d[i], wj, s);
     }
   }
   pw3[(size_t)c * H + j] = a;
