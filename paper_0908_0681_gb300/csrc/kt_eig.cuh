@@ -1037,12 +1037,16 @@ __global__ void __launch_bounds__(SOLO ? 128 : 256, SOLO ? 4 : 2)
   int *rs = sh.res_sgn + (SOLO ? 64 * wib : 0);
   double mx = -INFINITY, acc = 0.0;
   int wst = KT_OK;
-  if (MEAS)
-    for (int q = tid; q < nk; q += nt) ws.item_sign[(size_t)w * nk + q] = 0;
   for (int q0 = 0; q0 < nk; q0 += 64) {
     const int nq = min(64, nk - q0);
     const unsigned long long alive =
         BUILD ? (nq == 64 ? ~0ull : (1ull << nq) - 1) : eig_alive(M, cur, Kn, q0, nq, lane);
+    if (MEAS) {
+      // the pruned items count as zero; a surviving item's sign is written by its own warp only (nothing
+      // orders the warps before the reduction)
+      for (int q = tid; q < nq; q += nt)
+        if (!((alive >> q) & 1)) ws.item_sign[(size_t)w * nk + q0 + q] = 0;
+    }
     if (CACHE == EIG_RATIO && write) {
       // the commit of an accepted move needs the plan of the items that are zero now, too
       for (int q = tid; q < nq; q += nt)
