@@ -478,6 +478,25 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
     const double2 l = __ldcg((half ? C.blog : C.flog) + wk.entry);
     L0 = l.x - (l.y == 1.0 ? 0.0 : log(l.y));
   }
+  // CACHED: the group's states from operator number s0 of the half on are zero
+  auto store_zeros = [&](int s0) {
+    for (int s = s0 + gl; s < n; s += G) {
+      const int ij = half ? wk.i0 - s : wk.i0 + s;
+      const bool out = half ? ij >= wk.hi : ij + 1 <= wk.lo;
+      const size_t e = wk.eb + (half ? Kn - ij : ij + 1);
+      (half ? (out ? C.bblk : C.sbblk) : (out ? C.fblk : C.sfblk))[e] = -1;
+      (half ? (out ? C.blog : C.sblog) : (out ? C.flog : C.sflog))[e] = make_double2(0.0, 1.0);
+    }
+  };
+  if constexpr (CACHED) {
+    // A half that starts from a zero state stays zero, and its entry names no block: it follows no
+    // operators (block 0 and its key would lead to operators without a target, whose block -1 must
+    // never index a table) and stands on block 0 to the end.
+    if (u.vanished) {
+      if (wk.store) store_zeros(0);
+      n = 0;
+    }
+  }
   if constexpr (CACHED) {
     // the interval from a cached state to the first operator
     const bool act = on && wk.entry >= 0 && !u.vanished;
@@ -728,12 +747,7 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
     if constexpr (BUILD) {
       // every group's path has broken: the states that are left are zero
       if (__all_sync(FULL, u.vanished || base + G >= n)) {
-        if (wk.store && u.vanished)
-          for (int t = base + G + gl; t < n; t += G) {
-            const size_t e = wk.eb + 1 + t;
-            (half ? C.bblk : C.fblk)[e] = -1;
-            (half ? C.blog : C.flog)[e] = make_double2(0.0, 1.0);
-          }
+        if (wk.store && u.vanished) store_zeros(base + G);
         break;
       }
     }
