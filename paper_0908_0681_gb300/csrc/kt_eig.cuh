@@ -826,8 +826,10 @@ __device__ __forceinline__ unsigned long long eig_alive(const DevModel &M, const
   return nn != 0 || mk != 0 ? 0ull : alive;
 }
 
-// Overlap of the two halves of an item, its log-weight and sign (all lanes of half 0 hold them)
-// and, with MEAS, its observables at the meeting time into the workspace.
+// Overlap of the two halves of an item, its log-weight and sign (all lanes of half 0 hold them).
+// MEAS: into the workspace the matrix elements of the observables between the halves, their
+// overlap (half_log) and their common log-weight (item_log). The elements are not divided by the overlap:
+// a singlet and a triplet have none, but n_f and S_z have elements between them.
 template <int MODE, int G, int DMAX, bool MEAS, typename SH>
 __device__ __forceinline__ void eig_overlap(const DevModel &M, const Workspace &ws, SH &sh, EigHalf<MODE, G, DMAX> &u,
                                             bool on, int half, int item, double &L, int &sgn) {
@@ -897,13 +899,12 @@ __device__ __forceinline__ void eig_overlap(const DevModel &M, const Workspace &
       // n_f and double occupancies, one lane each
       const int nl = M.nf + M.n_orb + 1, off = __ldg(M.blk_off + u.b);
       double *io = ws.item_obs + (size_t)item * nl;
-      const double iov = zero ? 0.0 : 1.0 / ov;
       for (int k = gl; k < nl - 1; k += G) {
         const int bit = k < M.nf ? k : 2 * (k - M.nf), msk = k < M.nf ? 1 : 3;
         double a = 0.0;
         for (int r = 0; r < u.dim; ++r)
           if (((__ldg(M.st_bits + off + r) >> bit) & msk) == msk) a = fma(fv[r], bv[r], a);
-        io[k] = a * iov;
+        io[k] = a;
       }
       // S^2: sum_r backward_r (S^2 forward)_r
       const int s2w = __ldg(M.blk_s2w + u.b), s2o = __ldg(M.blk_s2ell + u.b);
@@ -920,10 +921,11 @@ __device__ __forceinline__ void eig_overlap(const DevModel &M, const Workspace &
 #pragma unroll
       for (int o = G / 2; o > 0; o >>= 1) a += __shfl_xor_sync(hm, a, o);
       if (gl == 0) {
-        io[nl - 1] = a * iov;
+        io[nl - 1] = a;
         ws.item_blk[item] = u.b;
-        ws.item_log[item] = L;
-        ws.item_sign[item] = (int8_t)sgn;
+        ws.item_log[item] = van ? -INFINITY : u.L + Lo;
+        ws.half_log[item] = ov;
+        ws.item_sign[item] = van ? 0 : 1;  // whether the item takes part
       }
     }
   }
@@ -1152,24 +1154,27 @@ __global__ void __launch_bounds__(SOLO ? 128 : 256, SOLO ? 4 : 2)
   wst = __reduce_max_sync(FULL, wst);
   if (lane == 0) eig_output(M, w, has_moves, cur_sign, cur_logabs, mx, acc, wst, sign, logv, status);
   if constexpr (MEAS) {
-    // the items' observables weighted by their share of the trace, and the (n_up, n_dn) histogram
+    // sums over the items of weight times element, in units of exp(mx), over the trace in the same units;
+    // the (n_up, n_dn) histogram adds the overlaps
     double *out = obs + (size_t)w * nobs;
-    const double inv = (acc != 0.0 && isfinite(mx)) ? 1.0 / acc : NAN;
+    const bool some = acc != 0.0 && isfinite(mx);
     for (int k = lane; k < nobs; k += 32) {
-      double a = 0.0;
+      double a = 0.0, den = 0.0;
       for (int q = 0; q < nk; ++q) {
         const int item = w * nk + q;
-        const int is = ws.item_sign[item];
-        if (is == 0) continue;
-        const double c = (double)is * exp(ws.item_log[item] - mx);
+        if (ws.item_sign[item] == 0) continue;
+        const double c = exp(ws.item_log[item] - mx), ov = ws.half_log[item];
+        double e = 0.0;
         if (k < nl) {
-          a = fma(c, ws.item_obs[(size_t)item * nl + k], a);
+          e = ws.item_obs[(size_t)item * nl + k];
         } else {
           const int x = __ldg(M.st_bits + __ldg(M.blk_off + ws.item_blk[item]));
-          if (__popc(x & 0x5555) * (M.n_orb + 1) + __popc(x & 0xaaaa) == k - nl) a += c;
+          if (__popc(x & 0x5555) * (M.n_orb + 1) + __popc(x & 0xaaaa) == k - nl) e = ov;
         }
+        if (e != 0.0) a = fma(c, e, a);    // c may be huge where both elements are zero
+        if (ov != 0.0) den = fma(c, ov, den);
       }
-      out[k] = a * inv;
+      out[k] = some ? a / (den != 0.0 ? den : acc) : NAN;
     }
   }
 }

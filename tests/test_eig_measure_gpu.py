@@ -15,6 +15,7 @@ if not torch.cuda.is_available():
     pytest.skip("no CUDA device", allow_module_level=True)
 
 from paper_0908_0681_gb300 import engine, kt, workloads  # noqa: E402
+from tests import test_eig_zero_states_gpu as ties, test_measure_gpu as measured  # noqa: E402
 
 
 def _walkers(w, n_long):
@@ -57,3 +58,17 @@ def test_every_item_counts(name, trunc_eps, n_long, prec):
         big = [t.cpu().numpy() for t in engine.measure(m, engine.DeviceSeqs.from_host(many))]
         for a, b in zip(first, big[:3]):
             assert np.array_equal(a[np.arange(2500) % seqs.n], b, equal_nan=a.dtype == np.float64)
+
+
+@pytest.mark.parametrize("prec", [kt.KT_FP64, kt.KT_FP32_KRYLOV])
+@pytest.mark.parametrize("n_orb", [3, 4])
+def test_halves_without_overlap(n_orb, prec):
+    """An item whose halves are a singlet and a triplet adds nothing to the trace, but n_f has an element
+    between them: the oracle's observables, with its tolerances. Operators at equal times project a
+    kept state on one orbital's occupation and leave such halves."""
+    lists = [[(0.5, 3, 0), (0.5, 3, 1), (0.9, 4, 1), (1.2, 4, 0), (2.0, 5, 1), (2.6, 5, 0)],
+             [(1.15, 1, 0), (1.75, 1, 1), (2.55, 0, 0), (2.85, 0, 1), (3.25, 3, 0), (3.25, 3, 1)],
+             [(0.5, 5, 0), (0.5, 5, 1), (0.9, 0, 0), (0.963, 0, 1), (0.971, 0, 0), (1.2, 0, 1), (2.0, 1, 0), (2.6, 1, 1)],
+             [(1.0, 0, 0), (1.0, 0, 1)], [(3.0, 1, 1), (3.0, 1, 0)], []]
+    lists += ties._batch(n_orb, 60, 13)[0]
+    measured.check(ties._spec(n_orb), ties._csr(lists), prec, f"{n_orb} orbitals, ties", min_regular=40)

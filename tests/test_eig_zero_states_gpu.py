@@ -5,7 +5,8 @@ one whose blocks hold orbital a singly occupied becomes exactly zero there, and 
 cached as zero. The edited window then holds two more operators at equal times. Four and seven orbitals
 have block counts that fill the model's tables to the last word (128 and 2,368 blocks). The cached
 results are compared with the calls from scratch, which start from the kept states: two evaluations
-of one ratio, each within RTOL of the exact value.
+of one ratio, each within RTOL of the exact value, and observables within the tolerances of
+tests/test_measure_gpu.py.
 """
 import numpy as np
 import pytest
@@ -19,6 +20,7 @@ from paper_0908_0681_gb300 import engine, kt, workloads  # noqa: E402
 from tests import parity  # noqa: E402
 
 BETA = 4.0
+OBS_ATOL = {kt.KT_FP64: 1e-9, kt.KT_FP32_KRYLOV: 3e-5}
 SPECS = {3: (0.0, 5.0), 4: (0.0, 8.0), 5: (1e-2, 13.0), 7: (3e-2, 24.0)}  # trunc_eps, mu: more than half filled
 
 
@@ -115,3 +117,29 @@ def test_ratios_and_commits(n_orb, count, prec):
         mv = workloads.Moves(np.zeros(count, np.uint8), mv.flavor ^ 1, np.full(count, 1.7 + 0.05 * step),
                              np.full(count, 2.3 + 0.05 * step), np.zeros(count, np.int32))
     assert hits > count // 4
+
+
+@pytest.mark.parametrize("prec", [kt.KT_FP64, kt.KT_FP32_KRYLOV])
+@pytest.mark.parametrize("n_orb,count", [(3, 600), (4, 300), (7, 60)])
+def test_observables_of_cached_chains(n_orb, count, prec):
+    """Each step's measurement starts from cached states; the accumulated increments against kt_measure."""
+    spec = _spec(n_orb)
+    m = engine.model_from_spec(spec, precision=prec)
+    lists, _ = _batch(n_orb, count, 5 * n_orb)
+    s = engine.trace(m, engine.DeviceSeqs.from_host(_csr(lists)))[0].cpu().numpy()
+    lists = [ops for ops, x in zip(lists, s) if x != 0]
+    assert len(lists) > count // 8
+    sw = engine.Sweep(m, workloads.semicircular_hybridization(BETA, 2 * n_orb, n_quad=256), BETA, len(lists), k_cap=16,
+                      n_bins=20, measure_obs=True, cache_ops=32)
+    sw.set_configs(_csr(lists))
+    g = torch.Generator(device="cuda").manual_seed(3)
+    last = sw.accumulators()["obs_sum"].cpu().numpy()
+    for _ in range(8):
+        sw.run(torch.rand((1, len(lists), 6), dtype=torch.float64, device="cuda", generator=g), meas_every=1)
+        now = sw.accumulators()["obs_sum"].cpu().numpy()
+        sign = sw.state()["sign"].cpu().numpy().astype(np.float64)
+        ref = engine.measure(m, engine.DeviceSeqs.from_host(_csr(sw.configs())))
+        want = ref[2].cpu().numpy() * sign[:, None]
+        # the sums before this step are at most 8 times the observables: their rounding is far below the bound
+        assert np.abs((now - last) - want).max() <= 2 * OBS_ATOL[prec] * max(1.0, np.abs(want).max())
+        last = now
