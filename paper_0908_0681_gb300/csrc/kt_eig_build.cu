@@ -10,13 +10,14 @@ namespace {
 using namespace dev;
 
 // Entry (r, k) of the matrix of c_f (dag 0) or c_f^+ (dag 1) from block b to its target: the sum
-// over the target's rows i with bit f equal to dag of V_t[i, r] (+-1) V_b[partner(i), k], in
-// FP64. Entries below 2^-42 are the eigensolver's rounding of exact (symmetry) zeros and are
-// stored as zeros: a component that a symmetry forbids then stays exactly zero, where the
-// propagator would amplify its rounding by exp(dt gap). (Measured on the five- and
-// seven-orbital models: entries of that origin end at 1e-13, the others start at 1e-10.)
+// over the target's rows i with bit f equal to dag of V_t[i, r] (+-1) V_b[partner(i), k], with vectors
+// and sum of two FP64 words each (kt_refine.h). An element that a symmetry of the model forbids
+// ends below the bound of its operator (eig_op.w, 1e-25 for the five-orbital model) and is stored as zero: a
+// component that a symmetry forbids then stays exactly zero, where the propagator would amplify
+// its rounding by exp(dt gap). Elements above it, however small, are the model's (weak hopping, weak
+// splitting) and are kept to the accuracy of their format.
 template <int MODE>
-__global__ void eig_matrix_kernel(DevModel M, typename EigT<MODE>::E *__restrict__ out) {
+__global__ void eig_matrix_kernel(DevModel M, const double *__restrict__ evec_lo, typename EigT<MODE>::E *__restrict__ out) {
   constexpr int EPV = EigT<MODE>::EPV;
   const int id = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (id >= M.n_blocks * M.nf * 2) return;
@@ -24,20 +25,32 @@ __global__ void eig_matrix_kernel(DevModel M, typename EigT<MODE>::E *__restrict
   if (e.z < 0) return;
   const int b = id / (2 * M.nf), f = (id >> 1) % M.nf, dag = id & 1;
   const int d1 = M.blk_dim[b], d2 = M.blk_dim[e.z], off = M.blk_off[e.z];
-  const double *V1 = M.blk_evec64 + M.blk_evoff[b], *V2 = M.blk_evec64 + M.blk_evoff[e.z];
+  const int o1 = M.blk_evoff[b], o2 = M.blk_evoff[e.z];
+  const double cut = (double)__int_as_float(e.w);
   const int ld = (d1 + EPV - 1) / EPV * EPV;
   typename EigT<MODE>::E *o = out + (size_t)e.x * EPV;
   for (int i = lane; i < d2 * ld; i += 32) {
     const int r = i / ld, k = i - r * ld;
-    double a = 0.0;
+    double a = 0.0, al = 0.0;
     if (k < d1)
       for (int s = 0; s < d2; ++s)
         if (((M.st_bits[off + s] >> f) & 1) == dag) {
           const unsigned pe = M.partner[(size_t)(off + s) * M.nf + f];
-          const double v = V2[r * d2 + s] * V1[k * d1 + (pe & 0x7fffu)];
-          a += (pe & 0x8000u) ? -v : v;
+          const int i2 = o2 + r * d2 + s, i1 = o1 + k * d1 + (int)(pe & 0x7fffu);
+          const double y = M.blk_evec64[i2], x = (pe & 0x8000u) ? -M.blk_evec64[i1] : M.blk_evec64[i1];
+          const double xl = (pe & 0x8000u) ? -evec_lo[i1] : evec_lo[i1];
+          const double p = __dmul_rn(y, x);
+          const double pl = fma(y, x, -p) + (y * xl + evec_lo[i2] * x);
+          // (a, al) += (p, pl)
+          const double t = a + p, bb = t - a;
+          const double te = (a - (t - bb)) + (p - bb);
+          const double u = al + pl, ub = u - al;
+          const double ue = (al - (u - ub)) + (pl - ub);
+          const double v = te + u, h = t + v, hl = (v - (h - t)) + ue;
+          a = h + hl;
+          al = hl - (a - h);
         }
-    if (fabs(a) < 2.3e-13) a = 0.0;
+    if (fabs(a) < cut) a = 0.0;
     if constexpr (MODE == EIG_PAIR) {
       const double h = rint(a * 2048.0) * (1.0 / 2048.0);
       o[i] = make_float2((float)h, (float)(a - h));
@@ -49,12 +62,12 @@ __global__ void eig_matrix_kernel(DevModel M, typename EigT<MODE>::E *__restrict
 
 }  // namespace
 
-int build_eig_matrices(const DevModel &M) {
+int build_eig_matrices(const DevModel &M, const double *evec_lo) {
   const unsigned grid = (unsigned)((M.n_blocks * M.nf * 2 + 7) / 8);
   void *o = const_cast<void *>(M.eig_mat);
   switch (M.eig) {
-    case EIG_PAIR: eig_matrix_kernel<EIG_PAIR><<<grid, 256>>>(M, (float2 *)o); break;
-    case EIG_F64: eig_matrix_kernel<EIG_F64><<<grid, 256>>>(M, (double *)o); break;
+    case EIG_PAIR: eig_matrix_kernel<EIG_PAIR><<<grid, 256>>>(M, evec_lo, (float2 *)o); break;
+    case EIG_F64: eig_matrix_kernel<EIG_F64><<<grid, 256>>>(M, evec_lo, (double *)o); break;
   }
   return (int)cudaGetLastError();
 }

@@ -64,7 +64,8 @@ struct DevModel {
   const int32_t *kept_key;    // [n_kept] the key of the kept state's block
   const int32_t *kept_row;    // [n_kept] its eigenvalue index inside the block
   const int4 *eig_op;         // [n_blocks * nf * 2] {first 16-byte vector of the matrix, blk_off of the target |
-                              //   rows of the source << 16 | rows of the target << 22, target, 0}
+                              //   rows of the source << 16 | rows of the target << 22, target,
+                              //   (float) bound below which an element is a zero}
   const double *eig_base;     // [n_blocks] s_b - E0
   const void *eig_lam;        // [n_states] (lambda_k - lambda_0) log2 e per global row: float pairs, or FP64
   const void *eig_tab;        // 2^(j/32) as 32 float pairs, or 2^(j/128) as 128 FP64
@@ -181,9 +182,9 @@ int launch_pipeline(const DevModel &m, int precision, int kernel_dmax, int group
                     kt_stats *stats, const Workspace &ws, void *stream, const StageEvents *timing,
                     double *obs = nullptr);
 
-// Operator matrices between the block eigenbases (eig_op, eig_mat) from the eigenvectors,
-// on the default stream. Returns a CUDA error code.
-int build_eig_matrices(const DevModel &m);
+// Operator matrices between the block eigenbases (eig_op, eig_mat) from the eigenvectors
+// blk_evec64 + evec_lo (DEVICE, the same layout), on the default stream. Returns a CUDA error code.
+int build_eig_matrices(const DevModel &m, const double *evec_lo);
 // The whole call in the block eigenbasis (m.eig >= 0), one kernel: arguments as launch_pipeline.
 int launch_eig_pipeline(const DevModel &m, int kernel_dmax, int group_lanes, const SeqView &seq, const MoveView *moves,
                         const int8_t *cur_sign, const double *cur_logabs, int8_t *sign, double *logv, int32_t *status,

@@ -11,14 +11,17 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <map>
 #include <new>
+#include <thread>
 #include <tuple>
 #include <vector>
 
 #include "kt_internal.h"
+#include "kt_refine.h"
 
 namespace {
 
@@ -83,6 +86,35 @@ void jacobi_eigh(int d, std::vector<double> A, std::vector<double> &w, std::vect
     for (int i = 0; i < d; ++i) Vs[(size_t)i * d + j] = V[(size_t)i * d + idx[j]];
   }
   V.swap(Vs);
+}
+
+// f(b) for every block, the blocks shared out to the cores where their d^3 operations would take
+// longer than starting threads (40 ns each: seven orbitals 115 ms on one core). False if memory ran out.
+template <typename F>
+bool for_each_block(const std::vector<int32_t> &dim, const F &f) {
+  std::atomic<int> next{0};
+  std::atomic<bool> ok{true};
+  const int B = (int)dim.size();
+  auto work = [&] {
+    try {
+      for (int b; (b = next++) < B;) f(b);
+    } catch (const std::bad_alloc &) {
+      ok = false;
+    }
+  };
+  double ops = 0.0;
+  for (const int d : dim) ops += (double)d * d * d;
+  std::vector<std::thread> pool;
+  try {
+    pool.reserve(16);
+    const int n = ops < 2e5 ? 1 : (int)std::min(16u, std::thread::hardware_concurrency());
+    for (int i = 1; i < n; ++i) pool.emplace_back(work);
+  } catch (const std::exception &) {
+    // no more threads: these and this one do
+  }
+  work();
+  for (auto &t : pool) t.join();
+  return ok;
 }
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -561,32 +593,76 @@ kt_status kt_model_create(const kt_model_params *pp, kt_model **out) {
                       : P.precision == KT_FP64 ? 1 : 0;  // EIG_F64, EIG_PAIR
   const int epv = 2;                 // matrix elements per 16-byte vector
   std::vector<int32_t> eig_op;       // int4 entries
-  std::vector<double> eig_base(B), eig_lam64, eig_tab64, evec64;
+  std::vector<double> eig_base(B), eig_lam64, eig_tab64, evec64, evec64lo, kept_e_dev = kept_e;
   std::vector<float> eig_lam32, eig_tab32;
   size_t eig_vecs = 0;
   if (eig >= 0) {
     M->group_lanes = kt::default_eig_group_for(M->kernel_dmax);
+    // H_loc's blocks and their eigenpairs in double-double: sums of the parameters are exact to 106
+    // bits, so what the model's symmetries make equal is equal
+    using kt::dd;
+    std::vector<std::vector<dd>> w2(B), v2(B);
+    std::vector<double> rest(B);
+    auto refine = [&](int b) {
+      const int d = blk_dim[b];
+      std::vector<dd> H((size_t)d * d);
+      for (int r = 0; r < d; ++r) {
+        const uint32_t x = members[b][r];
+        dd e(-blk_shift[b]);
+        for (int a = 0; a < n; ++a) {
+          const int u = (x >> (2 * a)) & 1, dn = (x >> (2 * a + 1)) & 1;
+          e = e - dd(u + dn) * kt::dd_sum(mu, M->delta[a]) + dd(u * dn) * dd(U);
+          for (int c = 0; c < a; ++c) {
+            const int cu = (x >> (2 * c)) & 1, cd = (x >> (2 * c + 1)) & 1;
+            e = e + dd(u * cd + dn * cu) * dd(Up) + dd(u * cu + dn * cd) * kt::dd_sum(Up, -J);
+          }
+        }
+        H[(size_t)r * d + r] = e;
+        for (auto &o : rows[x]) H[(size_t)r * d + o.first] = H[(size_t)r * d + o.first] + dd(o.second);
+      }
+      kt::refine_eigh(d, H, blk_norm[b], evecs[b], w2[b], v2[b]);
+      rest[b] = kt::refine_rest(d, blk_norm[b]) * std::sqrt((double)d);
+    };
+    if (!for_each_block(blk_dim, refine)) {
+      delete M;
+      return KT_ENOMEM;
+    }
+    for (int k = 0; k < NK; ++k) {
+      const int b = kept[k].b;
+      kept_e_dev[k] = (w2[b][kept[k].j] + kt::dd_sum(blk_shift[b], -E0)).h;
+    }
     eig_op.resize((size_t)B * nf * 2 * 4);
     for (size_t i = 0; i < (size_t)B * nf * 2; ++i) {
       const int b = (int)(i / (2 * nf)), t = blk_target[i];
       eig_op[4 * i] = (int32_t)eig_vecs;
       eig_op[4 * i + 1] = t < 0 ? 0 : blk_off[t] | blk_dim[b] << 16 | blk_dim[t] << 22;
       eig_op[4 * i + 2] = t;
-      eig_op[4 * i + 3] = 0;
+      // Elements below this are zeros of the model (eig_matrix_kernel). The off-diagonal rest mixes into an
+      // eigenvector a share rest / gap of each other one; gaps below 1 / beta cannot amplify it by
+      // more than e. The elements between two blocks have columns of norm 1 at most, which leaves
+      // beta rest sqrt(d) from each side, beside the rounding of the vectors and of the sums; with a
+      // factor of 16 for the roundings of the rotations.
+      const float cut = t < 0 ? 0.f : (float)(16.0 * (P.beta * (rest[b] + rest[t]) + std::ldexp(8.0 * (blk_dim[b] + blk_dim[t]), -104)));
+      std::memcpy(&eig_op[4 * i + 3], &cut, 4);
       if (t >= 0) eig_vecs += (size_t)blk_dim[t] * ((blk_dim[b] + epv - 1) / epv);
     }
-    const double log2e = 1.4426950408889634074;
+    const dd log2e(1.4426950408889634074, 2.0355273740931033e-17);
     for (int b = 0; b < B; ++b) {
-      eig_base[b] = blk_shift[b] - E0;
+      eig_base[b] = (w2[b][0] + kt::dd_sum(blk_shift[b], -E0)).h;
       for (int k = 0; k < blk_dim[b]; ++k) {
-        const double l = st_eval64[blk_off[b] + k] * log2e;
+        const dd gap = w2[b][k] - w2[b][0];
+        st_eval64[blk_off[b] + k] = gap.h;
+        const double l = (gap * log2e).h;
         if (eig == 1) {
           eig_lam64.push_back(l);
         } else {
           eig_lam32.push_back((float)l);
           eig_lam32.push_back((float)(l - (double)(float)l));
         }
-        for (int r = 0; r < blk_dim[b]; ++r) evec64.push_back(evecs[b][(size_t)r * blk_dim[b] + k]);
+        for (int r = 0; r < blk_dim[b]; ++r) {
+          evec64.push_back(v2[b][(size_t)k * blk_dim[b] + r].h);
+          evec64lo.push_back(v2[b][(size_t)k * blk_dim[b] + r].l);
+        }
       }
     }
     for (int j = 0; eig == 1 && j < 128; ++j) eig_tab64.push_back(std::exp2(j / 128.0));
@@ -610,7 +686,7 @@ kt_status kt_model_create(const kt_model_params *pp, kt_model **out) {
                i_d64 = add(st_diag64.data(), N * 8), i_d32 = add(st_diag32.data(), N * 4),
                i_ecol = add(ell_col.data(), ell_col.size() * 2), i_ev64 = add(ell_val64.data(), ell_val64.size() * 8),
                i_ev32 = add(ell_val32.data(), ell_val32.size() * 4), i_part = add(partner.data(), partner.size() * 2),
-               i_kb = add(kept_blk.data(), NK * 4), i_ke = add(kept_e.data(), NK * 8), i_ko = add(kept_off.data(), NK * 4),
+               i_kb = add(kept_blk.data(), NK * 4), i_ke = add(kept_e_dev.data(), NK * 8), i_ko = add(kept_off.data(), NK * 4),
                i_kv64 = add(kept_vec64.data(), kept_vec64.size() * 8), i_kv32 = add(kept_vec32.data(), kept_vec32.size() * 4),
                i_s2d = add(s2_diag_blk.data(), N * 4), i_s2e = add(s2_ell.data(), s2_ell.size() * 2),
                i_s2w = add(blk_s2w.data(), B * 4), i_s2o = add(blk_s2ell.data(), B * 4),
@@ -678,10 +754,20 @@ kt_status kt_model_create(const kt_model_params *pp, kt_model **out) {
     D.eig_mat = M->eig_mem;
     M->dev_bytes += bytes;
     // the caller may use the model on any stream at once: the matrices are complete on return
-    if (kt::build_eig_matrices(D) != 0 || cudaStreamSynchronize(0) != cudaSuccess) {
+    double *lo = nullptr;  // low halves of the eigenvectors, for the matrices only
+    kt_status rc = KT_OK;
+    if (cudaMalloc(&lo, evec64lo.size() * 8) != cudaSuccess) {
+      lo = nullptr;
+      rc = KT_ENOMEM;
+    } else if (cudaMemcpy(lo, evec64lo.data(), evec64lo.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess ||
+               kt::build_eig_matrices(D, lo) != 0 || cudaStreamSynchronize(0) != cudaSuccess) {
+      rc = KT_ECUDA;
+    }
+    if (lo) cudaFree(lo);
+    if (rc != KT_OK) {
       cudaGetLastError();
       kt_model_destroy(M);
-      return KT_ECUDA;
+      return rc;
     }
   }
   *out = M;
