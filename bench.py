@@ -9,15 +9,15 @@ tolerance 1e-12; 4,096 walkers with per-flavor orders Poisson(6) (capped at
 40); one proposed insert/remove move per walker per step (rounds of moves with
 seeds 1000 + r; the walkers' configurations are not advanced). A step is one
 trace-ratio evaluation of every walker's move: validation and move editing,
-structural pruning, the Krylov trace of every surviving (walker, kept state)
-pair and the reduction to sign and log-ratio. Inputs are resident in HBM; L2
+structural pruning, the trace of every surviving (walker, kept state) pair in
+the block eigenbasis and the reduction to sign and log-ratio, one kernel. Inputs are resident in HBM; L2
 is flushed (256 MiB write) before every timed step. Each rank runs its own
 4,096 walkers (weak scaling); there is no data-path collective.
 
-Prints one JSON line (rank 0). The FP32-Krylov path is the headline; the plain
+Prints one JSON line (rank 0). The FP32 path (KT_FP32_KRYLOV) is the headline; the plain
 FP64 GPU path is timed on the same rounds (key "fp64_gpu"). Key "sweep": full
 CT-HYB sweeps of the same model (semicircular bath, 1,024 chains, beta 50 by
-default) through kt_sweep, FP32-Krylov and FP64 traces.
+default) through kt_sweep, FP32 and FP64 traces; --details FILE has all of its figures.
 """
 from __future__ import annotations
 
@@ -67,6 +67,7 @@ def args_():
     p.add_argument("--no-seven", action="store_true", help="skip the seven-orbital sub-dict of the default run")
     p.add_argument("--workload", choices=["five_orbital", "seven_orbital"], default="five_orbital",
                    help="five_orbital (4,096 walkers, the headline) or seven_orbital (256 walkers)")
+    p.add_argument("--details", default=None, help="file for every figure of the run (JSON; the line has a summary of the sweeps)")
     p.add_argument("--trunc-eps", type=float, default=None,
                    help="truncation threshold of the outer trace (default: the workload's, 1e-10)")
     return p.parse_args()
@@ -122,6 +123,8 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(rows)}
 
 
+ROOFLINE_DEFINITION = ("one dense product of two blocks per propagated interval (kt_stats.intervals of a counted call "
+                       "times 2 d^2, the mean over the blocks) / time")
 ITEMS_SOURCES = ("kt_internal.h", "kt_device.cuh", "kt_eig.cuh", "kt_eig_f32.cu")
 
 
@@ -332,8 +335,8 @@ def sweep_beta_light(dev, beta: float, steps: int, seed: int):
     chains from Poisson(6) starts thermalise untimed with FP32 traces; from the same state
     `steps` steps are timed for FP32, FP32 with the partial-state cache and FP64 traces, measuring
     every 50 steps. Efficiencies at equal error cover double occupancy, the order, every n_f and
-    G(tau) on every bin. The step's roofline fraction counts the trace pipeline's algorithmic
-    Krylov flops (kt_stats.flops_alg over 50 untimed steps) against the FP32 peak."""
+    G(tau) on every bin. The step's roofline fraction counts the products of its trace ratios
+    (ROOFLINE_DEFINITION, intervals of 50 untimed steps) against the FP32 peak."""
     import numpy as np
     import torch
 
@@ -389,7 +392,7 @@ def sweep_beta_light(dev, beta: float, steps: int, seed: int):
         sw.run(u[:50])
         sw.set_stats(None)
         wk = kt.stats_from_tensor(wst)
-        flops_step = wk["flops_alg"] / 50
+        flops_step = wk["intervals"] / 50 * 2 * mean_block_square(spec.n_orb)
         props = nw * steps / (ms / 1000.0)
         out[name] = {"proposals_per_s": props, "ms_per_step": ms / steps, "sweeps_per_s": props / K,
                      "mean_ops_per_chain": K, "mean_order_per_flavor": stt["order"].double().mean().item(),
@@ -401,7 +404,7 @@ def sweep_beta_light(dev, beta: float, steps: int, seed: int):
                      "roofline": {"bound": "alu", "achieved": flops_step / (ms / steps / 1000.0) / 1e12,
                                   "peak": peak32, "unit": "TFLOP/s",
                                   "frac": flops_step / (ms / steps / 1000.0) / 1e12 / peak32,
-                                  "definition": "algorithmic Krylov flops of the step's trace ratios / step time"}}
+                                  "definition": ROOFLINE_DEFINITION}}
         del sw
     sp = {f"{a_}_over_{b_}": speedups(eff[a_], eff[b_]) for a_, b_ in (("fp32", "fp64"), ("fp32_cached", "fp64"),
                                                                         ("fp32_cached", "fp32"))}
@@ -410,7 +413,7 @@ def sweep_beta_light(dev, beta: float, steps: int, seed: int):
 
 
 def seven_bench(dev, K: int):
-    """The seven-orbital batch (256 walkers, N_tr = 63, beta 40): FP32-Krylov and FP64
+    """The seven-orbital batch (256 walkers, N_tr = 63, beta 40): FP32 and FP64
     trace-ratio evaluations per second (L2 flushed before every step) and the largest relative
     error of each path's ratios, formed against its own current traces, against the oracle's
     ratios on the first round."""
@@ -477,9 +480,9 @@ def seven_bench(dev, K: int):
 def sweep_bench(dev, steps: int, beta: float, seed: int):
     """Full CT-HYB sweeps of the five-orbital model (semicircular bath, 2,000 tau points,
     1,024 chains). Chains start from Poisson(6) configurations and thermalise untimed
-    (FP32-Krylov traces). The surrogate is trained on the chains' own ratios
+    (FP32 traces). The surrogate is trained on the chains' own ratios
     (kt_sweep_collect, then Adam on the tensor cores). From the same thermalised state,
-    `steps` Metropolis steps are then timed with CUDA events for plain FP32-Krylov
+    `steps` Metropolis steps are then timed with CUDA events for plain FP32
     sweeps, delayed-acceptance FP32 sweeps and plain FP64 sweeps,
     measuring G(tau), the orders and the beta/2 observables every 50 steps.
 
@@ -612,7 +615,7 @@ def sweep_bench(dev, steps: int, beta: float, seed: int):
         gmid = (acc["g_tau"][:, :, 95:105].mean(2) * (200 / beta ** 2) / ssum[:, None]).mean(1)
         K = stt["lens"].double().mean().item()
         effs[name] = efficiencies(chain_estimates(acc, spec.n_orb, beta, 200), ms / 1000.0)
-        # algorithmic Krylov flops of the trace pipeline per step (50 untimed steps)
+        # intervals of the step's trace ratios (50 untimed, counted steps)
         wst = engine.new_stats(dev)
         sw.set_stats(wst)
         if mode == "multi":
@@ -622,7 +625,7 @@ def sweep_bench(dev, steps: int, beta: float, seed: int):
         else:
             sw.run(u[:50])
         sw.set_stats(None)
-        flops_step = kt.stats_from_tensor(wst)["flops_alg"] / 50
+        flops_step = kt.stats_from_tensor(wst)["intervals"] / 50 * 2 * mean_block_square(spec.n_orb)
         del sw
         per_chain[name] = {"docc": docc, "order": order, "G_beta_half": gmid,
                            "n_f": obs[:, :2 * spec.n_orb].mean(1), "S2": obs[:, 3 * spec.n_orb],
@@ -649,8 +652,8 @@ def sweep_bench(dev, steps: int, beta: float, seed: int):
                      "error_bars_binning": binning,
                      "roofline": {"bound": "alu", "achieved": flops_step / (ms / n_t / 1000.0) / 1e12, "peak": peak32,
                                   "unit": "TFLOP/s", "frac": flops_step / (ms / n_t / 1000.0) / 1e12 / peak32,
-                                  "flops_alg_per_step": flops_step,
-                                  "definition": "algorithmic Krylov flops of the step's trace ratios / step time"}}
+                                  "flops_per_step": flops_step,
+                                  "definition": ROOFLINE_DEFINITION}}
     # FP32 against FP64 on the same uniforms: chains whose final configurations agree took
     # the same decisions all along, so their accumulators differ only by the trace arithmetic
     a32, a64 = per_chain["fp32"], per_chain["fp64"]
@@ -816,6 +819,43 @@ def sweep_bench(dev, steps: int, beta: float, seed: int):
                           "target_std": spread, "network": "n_in-256-256-1 ReLU, BF16 tcgen05, FP32 accumulate"}}
 
 
+def brief(x, digits: int = 6):
+    """x with its floats rounded to `digits` significant digits."""
+    if isinstance(x, float):
+        return float(f"{x:.{digits}g}") if math.isfinite(x) else x
+    if isinstance(x, dict):
+        return {k: brief(v, digits) for k, v in x.items()}
+    return [brief(v, digits) for v in x] if isinstance(x, list) else x
+
+
+def brief_sweep(s):
+    """The sweep's rates and speedups: sweep_bench's own dict is about 37,000 characters."""
+    if s is None:
+        return None
+
+    def rates(d):
+        return {m: {k: v[k] for k in ("proposals_per_s", "ms_per_step", "acceptance") if k in v}
+                for m, v in d.items() if isinstance(v, dict) and "proposals_per_s" in v}
+
+    out = {k: s[k] for k in ("workload", "metric", "measure_every", "speedup_fp32_over_fp64") if k in s}
+    out.update(rates(s))
+    out["speedup_at_equal_error_docc"] = {k: v["docc"] for k, v in s.get("speedup_at_equal_error", {}).items()}
+    if "throughput_8192_chains" in s:
+        out["throughput_8192_chains"] = {m: v["proposals_per_s"] for m, v in rates(s["throughput_8192_chains"]).items()}
+    for b, v in s.get("other_betas", {}).items():
+        out[b] = {m: r["proposals_per_s"] for m, r in rates(v).items()}
+    return out
+
+
+def printed_line(line):
+    """The line printed: the contract's numbers in full, the others to six digits, the sweep as its rates. It
+    stays below 8,192 characters, so that a reader of the last few kilobytes of the output gets it whole."""
+    full = ("value", "ms_per_step", "e2e", "clocks")
+    out = {k: v if k in full else brief(v) for k, v in line.items()}
+    out["sweep"] = brief(brief_sweep(line.get("sweep")))
+    return out
+
+
 def main():
     global DA_TRIES
     a = args_()
@@ -904,7 +944,7 @@ def main():
     K64 = a.fp64_steps if a.fp64_steps > 0 else min(a.steps, 100)
     ms64, stage64, _ = timed_loop(m64, cur64, K64, a.warmup)
 
-    # FP32 Krylov vectors with the final tridiagonal exponential to FP64 accuracy (KT_FP32_TRIDIAG64)
+    # the same with KT_FP32_TRIDIAG64, which changes Krylov propagations only
     m32t = engine.model_from_spec(w.model, precision=kt.KT_FP32_KRYLOV, flags=kt.KT_FP32_TRIDIAG64)
     tuned["fp32_tridiag64"] = kt.kt_autotune(m32t, dseq.batch(), out_s, out_l, out_st, ws)
     cur32t = current(m32t)
@@ -1045,9 +1085,8 @@ def main():
     value32t = n * Kt / (sum(ms32t) / 1000.0)
     tridiag = {"value": value32t, "unit": UNIT, "ms_per_step": sum(ms32t) / Kt, "steps": Kt,
                "speedup_over_fp64": value32t / value64, "flag": "KT_FP32_TRIDIAG64",
-               "precision": "FP32 Krylov vectors, tridiagonal exponential to FP64 accuracy (p = 2 closed form "
-                            "in FP64; p >= 3 FP32 Ritz vectors with one double-float refinement step and FP64 "
-                            "weights, FP64 QL where Ritz values are too close)"}
+               "precision": "as the default: the flag changes Krylov propagations only, and this model's blocks "
+                            "(at most 36 rows) are not propagated that way"}
     e2e_value = world * n / (e2e_ms / 1000.0)
 
     # roofline of the kernel of a ratio call (block eigenbasis)
@@ -1063,9 +1102,7 @@ def main():
     roofline = {"bound": "alu", "achieved": ach32, "peak": peak32, "unit": "TFLOP/s", "frac": ach32 / peak32,
                 "traffic": measured_traffic(sha), "kernel": "eig_kernel", "pipe": "fp32",
                 "flops_per_launch": f32_per_launch,
-                "flops_definition": "propagated intervals (kt_stats.intervals) times 2 d^2, the mean over the blocks",
-                "reorth_flops_per_launch": st["flops_reorth"] / a.steps,
-                "device_flops_vec_per_launch": st["flops_vec"] / a.steps,
+                "flops_definition": ROOFLINE_DEFINITION,
                 "items_ms_per_launch": items_ms,
                 "stage_ms_per_step": {k: v / max(nl32, 1) for k, v in stage32.items()},
                 "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 flops x max SM clock (sampled)",
@@ -1112,7 +1149,8 @@ def main():
                          "speedup_fp32_over_fp64": value / value64},
             "work": {"items_alive_per_step": st["items_alive"] / a.steps, "intervals_per_step": st["intervals"] / a.steps,
                      "mean_krylov_dim": st["krylov_iters"] / max(st["intervals"], 1), "p_max": st["p_max"],
-                     "noconv": st["noconv"], "flops_alg_per_step": f32_per_launch,
+                     "noconv": st["noconv"], "counted_by": "an untimed call with kt_stats (the Krylov route on the same inputs)",
+                     "flops_per_step": f32_per_launch,
                      "nonzero_fraction": nonzero_frac,
                      "value_over_nonzero_proposals": value * nonzero_frac,
                      "p_hist_fp32": trim_hist(st["p_hist"]), "p_hist_fp64": trim_hist(st64["p_hist"]),
@@ -1130,7 +1168,10 @@ def main():
             "gpu_launches": a.steps,
             "kernel_source_sha": sha,
         }
-        print(json.dumps(line), flush=True)
+        if a.details:
+            with open(a.details, "w") as f:
+                json.dump(line, f)
+        print(json.dumps(printed_line(line)), flush=True)
     if world > 1:
         torch.distributed.destroy_process_group()
 
