@@ -61,9 +61,17 @@ typedef enum {
 } kt_status;
 
 /* precision */
-#define KT_FP64 0         /* FP64 Krylov vectors and scalars (plain FP64 path) */
-#define KT_FP32_KRYLOV 1  /* FP32 SpMV and Krylov vectors; FP64-accurate (double-float)
-                             Lanczos scalars, norms and Ritz values; FP64 log-weights */
+#define KT_FP64 0         /* FP64 vectors and scalars (plain FP64 path) */
+#define KT_FP32_KRYLOV 1  /* FP32 vectors, FP64 log-weights. Block-eigenbasis route: pairs of floats.
+                             Krylov route: FP32 SpMV and Krylov vectors, FP64-accurate (double-float)
+                             Lanczos scalars, norms and Ritz values */
+
+/* Routes. Models whose blocks have at most 36 rows are evaluated in the eigenbasis of their blocks:
+ * an operator is a dense block-to-block product and an interval one exponential per component.
+ * Larger blocks (KT_SECTOR_BLOCKS beyond four orbitals), a krylov_pmax below the block size, and
+ * every call that counts its work (kt_stats) take the Krylov route: Lanczos propagation
+ * of each interval. krylov_tol, KT_FP32_TRIDIAG64 and KT_ENOCONV belong to the Krylov route and have no
+ * effect on the other. Both evaluate the same traces; they differ by rounding. */
 
 /* flags */
 #define KT_DENSITY_ONLY 1u   /* drop spin-flip and pair-hopping (density-density H_loc) */
@@ -80,8 +88,8 @@ typedef enum {
                                 35, 2018) in double-float, Ritz values recomputed from them and FP64
                                 weights; a T_p with Ritz values too close to refine takes a full
                                 FP64 QL. Exact stops: double-float sums over the block
-                                eigendecomposition. Slower than the default (the FP64 pipe of
-                                GB300 is 1/64 of the FP32 one) */
+                                eigendecomposition. Slower than the default there (the FP64 pipe of
+                                GB300 is 1/64 of the FP32 one). No effect in the block eigenbasis */
 #define KT_HOST_ONLY 256u    /* build and check the model on the host only: no device upload;
                                 trace calls on such a model return KT_EINVAL */
 
@@ -98,8 +106,9 @@ typedef struct {
   double trunc_eps;     /* keep whole multiplets with exp(-beta (E - E0)) >= trunc_eps;
                            <= 0 keeps every eigenstate (untruncated trace) */
   double deg_tol;       /* eigenvalues within deg_tol * max(1, |E|) form one multiplet */
-  double krylov_tol;    /* relative a-posteriori error target per propagation */
-  int32_t krylov_pmax;  /* cap on the Krylov dimension (<= 0: the compiled maximum) */
+  double krylov_tol;    /* relative a-posteriori error target per propagation (Krylov route) */
+  int32_t krylov_pmax;  /* cap on the Krylov dimension (<= 0: the compiled maximum); below the
+                           block size (and that maximum) it selects the Krylov route */
   int32_t precision;    /* KT_FP64 or KT_FP32_KRYLOV */
   uint32_t flags;       /* KT_DENSITY_ONLY | KT_SECTOR_BLOCKS | KT_FP32_TRIDIAG64 */
 } kt_model_params;
@@ -124,7 +133,10 @@ typedef struct {
 #define KT_P_HIST 32
 
 /* Per-call counters, accumulated on the device with atomics into a caller-owned
- * DEVICE struct (zero it before the call; pass NULL to skip counting). */
+ * DEVICE struct (zero it before the call; pass NULL to skip counting). A counted call takes the
+ * Krylov route and the counters describe that route's work, also where the call without
+ * them runs in the block eigenbasis; items and items_alive are the same for both. Results differ from an uncounted call's by rounding, so a counted sweep may decide
+ * a move at the edge of acceptance differently. */
 typedef struct {
   unsigned long long walkers;        /* walkers evaluated */
   unsigned long long items;          /* (walker, kept state) pairs */
@@ -354,9 +366,9 @@ void kt_ratio_cache_destroy(kt_ratio_cache *c);
  *
  * Partial-state cache (cache_ops > 0; Sec. III's forward and backward propagation,
  * kept between steps). For every walker and kept state the sweep stores, for its
- * current configuration of K operators, the normalised forward states after each
- * operator (times their log-weights) and the backward states from beta down to each
- * operator, each over a valid prefix and suffix of positions. A proposal edits the
+ * current configuration of K operators, the forward states after each
+ * operator (vectors of FP64, or of single floats on the FP32 path, with their log-weights) and the
+ * backward states from beta down to each operator, each over a valid prefix and suffix of positions. A proposal edits the
  * window between its first and last changed operator; its trace ratio propagates
  * only from the last valid forward state before the window to the first valid
  * backward state after it (split in the middle, forward and backward concurrently),
@@ -579,8 +591,8 @@ kt_status kt_sweep_run_da(kt_sweep *s, int32_t n_steps, const double *uniforms, 
 kt_status kt_sweep_run_da_multi(kt_sweep *s, int32_t n_steps, int32_t tries, const double *uniforms,
                                 int32_t meas_every, void *stream);
 
-/* Kernel tiling: every (walker, kept state) item of the Krylov stage is
- * processed by a group of group_lanes lanes of one warp (32 / group_lanes items
+/* Kernel tiling: every half of a (walker, kept state) item is
+ * processed by a group of group_lanes lanes of one warp (32 / group_lanes halves
  * per warp). kt_model_set_tiling picks one of the compiled group sizes
  * (KT_EINVAL if it is not compiled for this model's block size).
  * kt_autotune times kt_trace on the caller's batch (DEVICE buffers as in
@@ -594,7 +606,9 @@ kt_status kt_autotune(kt_model *m, const kt_seq_batch *batch, int8_t *sign, doub
  * After kt_timing_begin(m, max_launches), each of the next max_launches trace
  * or trace-ratio calls on m records CUDA events on its own stream around its
  * four stages: 0 validation/edit, 1 structural pruning and the ordering of the
- * surviving items by length (two kernels), 2 Krylov items, 3 reduction. kt_timing_end waits for those events, writes the summed
+ * surviving items by length (two kernels), 2 items, 3 reduction. A call in the block
+ * eigenbasis is one kernel, all of it in stage 2; its other stages hold the gaps between
+ * events (about 2 us each). kt_timing_end waits for those events, writes the summed
  * durations in milliseconds to ms_per_stage[4] and the number of recorded calls
  * to *launches, and stops recording. Calls beyond max_launches run untimed.
  * Not thread-safe: do not share a model between host threads while timing. */

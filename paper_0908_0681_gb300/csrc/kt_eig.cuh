@@ -24,12 +24,15 @@ namespace dev {
 
 // How a unit's vector is held. EIG_F64: FP64. EIG_PAIR, the FP32 path: a component x is a pair of
 // floats, x = h + l with h a multiple of 2^-10 and |l| <= 2^-11, and a matrix entry a pair with h
-// a multiple of 2^-11. The vector's norm stays below 8 and its largest component above 2^-8, so
-// the products h h and their sums over a row are exact in FP32, and the three other products
-// are summed in FP32 where they are 2^-11 smaller: 33 bits or more for four FMAs a term. Plain
-// FP32 components had an error of 4.7e-7 rms in log|T| at five orbitals, but up to 1.7e-5 where
-// a trace cancels and 2.5e-5 at seven orbitals; pairs with TwoSum sums (12 operations a term)
-// gave no smaller errors that a float could show.
+// a multiple of 2^-11. The vector's norm stays below 8, so the products h h and their sums over a
+// row are exact in FP32, and the three other products are summed in FP32 where they are 2^-11
+// smaller: an absolute error near 2^-34 for four FMAs a term. That is 33 bits of a vector of size 1,
+// 30 of one whose largest component is 1/16 (below it the next interval scales by 16) and 26 at 2^-8,
+// where it is scaled at once. A cached state is rounded to one float per component: errors of cached
+// log-ratios 3.2e-8 rms, 1.3e-7 at most at five orbitals (4,096 walkers), against 1.7e-9 and 1.7e-8
+// from scratch. Plain FP32 components throughout had an error of 4.7e-7 rms in log|T| at five
+// orbitals, but up to 1.7e-5 where a trace cancels and 2.5e-5 at seven orbitals; pairs with TwoSum
+// sums (12 operations a term) gave no smaller errors that a float could show.
 constexpr int EIG_PAIR = 0, EIG_F64 = 1;
 
 template <int MODE>
@@ -318,8 +321,9 @@ __device__ __forceinline__ bool eig_interval(const DevModel &M, typename EigT<MO
   return alive;
 }
 
-// EIG_PAIR, blocks of at most 12 rows: the same with the three small products in sums of their own, which
-// leaves chains of two FMAs a vector where one sum makes a chain of six.
+// One 16-byte vector of a row (two entries) times the vector in shared memory, EIG_PAIR, blocks of at most
+// 12 rows. a[0] collects the exact products of the first parts; the three small products have sums of
+// their own, chains of two FMAs a vector where eig_fma's one sum makes a chain of six.
 __device__ __forceinline__ void eig_fma4(float (&a)[4], const float4 &m, const float4 &v) {
   a[0] = fmaf(m.x, v.x, a[0]);
   a[1] = fmaf(m.x, v.y, a[1]);
@@ -352,7 +356,7 @@ __device__ __forceinline__ void eig_fma(typename EigT<MODE>::E &acc, const float
 }
 
 // Operators at equal times (code = 2 f + dag, from block bs to bt): between them the vector stays
-// in the occupation basis, where c_f and c_f^+ are gathers and exact zeros stay exact. x holds
+// in the occupation basis, where c_f and c_f^+ are gathers and exact zeros stay exact.
 // xs[cb] holds the vector (components, or rows when `fock`); the result's rows go to xs[cb] and
 // its components to xs[cb ^ 1]. `on`: the group has such an operator; all lanes of the warp call
 // it together. Continuous times never coincide, so this is kept small, in FP64.
@@ -1123,7 +1127,6 @@ __global__ void __launch_bounds__(SOLO ? 128 : 256, SOLO ? 4 : 2)
           wk.entry = (long long)(wk.eb + (half ? Kn - x : y));
           wk.t0 = cur.get(half ? x : y - 1).t;
         }
-        m = CACHE == EIG_RATIO ? me : m;
       }
       H u;
       eig_half<MODE, G, DMAX, CACHE != EIG_PLAIN, BUILD>(M, cur, Kn, wk, C, xs, u);

@@ -124,9 +124,10 @@ struct Workspace {
 // tau = 0 and is not stored) and backward states at reverse slot K - e (the bra
 // including operators e .. K-1, at the time of operator e; reverse slot 0 is the kept
 // state at beta). Entries are vectors with a log-weight and their block (-1: the state is
-// zero): components on the block's eigenvectors for models with traces in the block
-// eigenbasis (DevModel.eig >= 0), normalised vectors in the occupation basis otherwise. f[item] and gr[item] bound the valid forward slots
-// [0, f] and reverse slots [0, gr]. The scratch arrays hold one step's tentative
+// zero): components on the block's eigenvectors, of any norm, for models with traces in the
+// block eigenbasis (DevModel.eig >= 0), normalised vectors in the occupation basis
+// otherwise. f[item] and gr[item] bound the valid forward slots [0, f] and reverse slots
+// [0, gr]. The scratch arrays hold one step's tentative
 // states (inside the edited window) until the accept decision.
 struct CacheView {
   int P;              // positions per direction; walkers with more operators are not cached

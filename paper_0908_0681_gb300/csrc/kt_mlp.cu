@@ -97,7 +97,7 @@ __device__ __forceinline__ void stage_tile(uint8_t *dst, const __nv_bfloat16 *sr
 // What a tile's epilogue makes of the accumulator. The network's layers apply their bias, ReLU, mask and
 // rounding here, on the values in registers: as kernels of their own over the FP32 matrices
 // (bias and ReLU, masks, transposes, 4,096 x 256 values each) they and the small sums were 19 of a training
-// step's 24 launches, which are ten now: an epoch of eight 4,096-row steps 2,400 -> 884 us with all of it.
+// step's 24 launches, which are nine now: an epoch of eight 4,096-row steps 2,400 -> 880 us with all of it.
 //   EPI_STORE  C = acc
 //   EPI_ACT1   H1 = bf16(relu(acc + bias)), with C the FP32 acc too, with hT the transpose too
 //   EPI_OUT    y = v . relu(acc + bias) + *vb, for tiles that hold whole rows (N = 256 = BN)
