@@ -82,7 +82,9 @@ __device__ __forceinline__ void key_scan(int &nn, int &mk, int gl) {
 }
 
 // ---------------------------------------------------------------------------
-// 2^(-dt lambda2) of one component, lambda2 = (lambda_k - lambda_0) log2 e
+// 2^(-dt lambda2) of one component, lambda2 = (lambda_k - lambda_0) log2 e: reduction to the nearest entry
+// of a table of powers of two and a Taylor series of the rest (the table-driven method of P. T. P. Tang,
+// ACM Trans. Math. Softw. 15, 1989)
 // ---------------------------------------------------------------------------
 struct EigDt {
   float h, l;   // EIG_PAIR: dt as a pair
