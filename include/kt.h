@@ -282,7 +282,7 @@ kt_status kt_trace_ratio_static(kt_model *m, const kt_seq_batch *cur, const int8
 /* ------------------------------------------------------------------------ */
 /*
  * For fixed current configurations evaluated against many proposed updates,
- * kt_ratio_cache_build stores, for every walker and kept state, the normalised
+ * kt_ratio_cache_build stores, for every walker and kept state, the
  * forward state after each operator and the backward state from beta down to each
  * operator, with their log-weights. kt_trace_ratio_cached then propagates only the
  * window that an update edits: from the cached forward state before its first

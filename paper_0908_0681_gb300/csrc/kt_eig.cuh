@@ -439,8 +439,9 @@ struct EigWork {
 // The lanes of a group take one operator each of the next G (its block from the key prefixes,
 // its matrix, its interval), then the group walks through them. Every group of the warp makes
 // the same number of turns, so that all warp primitives are converged. CACHED: halves that start
-// from or store to the partial-state cache; BUILD: the block path may break (the states from
-// there on are stored as zero).
+// from or store to the partial-state cache. Their block path may break, in a BUILD because it covers items
+// that pruning would remove, else because the caller's sequences are not the cached ones: the states from
+// there on are zero.
 template <int MODE, int G, int DMAX, bool CACHED, bool BUILD>
 __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, int Kn, const EigWork &wk,
                                          const CacheView &C, typename EigT<MODE>::E *xs, EigHalf<MODE, G, DMAX> &u) {
@@ -580,7 +581,7 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
     if (have) {
       const int b = key_block(M, nn + pn - dn, mk ^ pm ^ dm);
       int4 e = make_int4(0, 0, -1, 0);
-      if (!BUILD || b >= 0) e = __ldg(M.eig_op + (size_t)max(b, 0) * 2 * M.nf + code);
+      if (!CACHED || b >= 0) e = __ldg(M.eig_op + (size_t)max(b, 0) * 2 * M.nf + code);
       moff = e.x;
       pk = e.y;
       tgt = e.z;
@@ -593,8 +594,8 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
     }
     nn += __shfl_sync(FULL, pn, G - 1, G);
     mk ^= __shfl_sync(FULL, pm, G - 1, G);
-    int dead = G;  // BUILD: the first of these operators without a target block
-    if constexpr (BUILD) {
+    int dead = G;  // CACHED: the first of these operators without a target block
+    if constexpr (CACHED) {
       const unsigned bad = __ballot_sync(FULL, have && tgt < 0) >> (lane / G * G);
       const unsigned gb = G == 32 ? bad : bad & ((1u << (G & 31)) - 1u);
       if (gb) dead = __ffs(gb) - 1;
@@ -618,8 +619,8 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
     bool vj = false;
     if constexpr (PRE) fetch(__shfl_sync(FULL, moff, 0, G), __shfl_sync(FULL, pk, 0, G));
     for (int j = 0; j < cnt; ++j) {
-      if (BUILD && j >= dead) u.vanished = true;
-      const bool act = base + j < n && !(BUILD && u.vanished);
+      if (CACHED && j >= dead) u.vanished = true;
+      const bool act = base + j < n && !(CACHED && u.vanished);
       const int mo = __shfl_sync(FULL, moff, j, G), pj = __shfl_sync(FULL, pk, j, G);
       EigDt dj{0.f, 0.f, 0.0};
       if constexpr (MODE == EIG_F64) {
@@ -749,7 +750,7 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
     }
     const int last = min(n - base, G) - 1;  // the block after the group's last operator so far
     const int tl = __shfl_sync(FULL, tgt, max(last, 0), G);
-    if (last >= 0) u.b = tl;
+    if (last >= 0) u.b = CACHED ? max(tl, 0) : tl;
     if constexpr (BUILD) {
       // every group's path has broken: the states that are left are zero
       if (__all_sync(FULL, u.vanished || base + G >= n)) {
@@ -758,7 +759,12 @@ __device__ __forceinline__ void eig_half(const DevModel &M, const Cursor &cur, i
       }
     }
   }
-  if constexpr (!CACHED) {
+  if constexpr (CACHED) {
+    if (u.vanished) {  // no block of its own
+      u.b = 0;
+      u.dim = __ldg(M.blk_dim);
+    }
+  } else {
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) Ll += __shfl_xor_sync(FULL, Ll, o);
   }

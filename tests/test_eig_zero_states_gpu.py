@@ -143,3 +143,23 @@ def test_observables_of_cached_chains(n_orb, count, prec):
         # the sums before this step are at most 8 times the observables: their rounding is far below the bound
         assert np.abs((now - last) - want).max() <= 2 * OBS_ATOL[prec] * max(1.0, np.abs(want).max())
         last = now
+
+
+@pytest.mark.parametrize("prec", [kt.KT_FP64, kt.KT_FP32_KRYLOV])
+@pytest.mark.parametrize("n_orb,count", [(4, 240), (4, 2600), (7, 48)])
+def test_a_stale_cache_stays_in_bounds(n_orb, count, prec):
+    """Sequences of the cached lengths but not the cached ones: a half's block path breaks, which counts as a
+    zero. The values mean nothing; after a build for the new sequences they are those from scratch again."""
+    m, m64 = engine.model_from_spec(_spec(n_orb), precision=prec), engine.model_from_spec(_spec(n_orb))
+    one, zero = torch.ones(count, dtype=torch.int8, device="cuda"), torch.zeros(count, dtype=torch.float64, device="cuda")
+    old, _ = _batch(n_orb, count, 1)
+    new, mv = _batch(n_orb, count, 2)
+    cache = engine.RatioCache(m, count, max_ops=16)
+    cache.build(engine.DeviceSeqs.from_host(_csr(old)))
+    d, dm = engine.DeviceSeqs.from_host(_csr(new)), engine.DeviceMoves.from_host(mv)
+    for call in (cache.ratio, cache.propose):
+        sign, log, status = (t.cpu().numpy() for t in call(d, one, zero, dm))
+        assert np.isin(sign, (-1, 0, 1)).all() and ((status == kt.KT_OK) | (status == kt.KT_ENUMERIC)).all()
+    cache.build(d)
+    call = (d, one, zero, dm)
+    _same((m64, call), engine.trace_ratio(m, *call), cache.ratio(*call), prec)
